@@ -44,7 +44,6 @@ struct hough_batch {
     HitInputs inputs_on_device{};        // what inputs_dev holds (copied only when it changes)
     float *in_r = nullptr, *in_phi = nullptr, *in_z = nullptr;
     uint8_t *in_layer = nullptr;
-    hough_candidate *packed = nullptr;   // all events' candidates, concatenated
     cudaStream_t capture_stream = nullptr;
     std::map<int, cudaGraphExec_t> graphs;   // by batch size
     int n_events = 0;                        // of the last run
@@ -135,10 +134,9 @@ int hough_batch_create(const hough_geometry *geometry, const hough_binning *binn
     A(b->alloc(&w.M, (size_t)E * ax.n_qpt * ax.n_phi));
     A(b->alloc(&w.band_cands, (size_t)E * band_list_entries(ax)));
     A(b->alloc(&w.band_counts, (size_t)E * n_bands(ax, 1))); A(b->alloc(&w.band_offs, (size_t)E * n_bands(ax, 1)));
-    A(b->alloc(&w.cands, E * C));
+    A(b->alloc(&w.cands, E * C)); A(b->alloc(&w.cand_list, E * C));
     A(b->alloc(&w.cand_base, E + 1)); A(b->alloc(&w.counters, 1));
     A(b->alloc(&w.stats, E));
-    A(b->alloc(&b->packed, E * C));
     if (e != cudaSuccess) {
         delete b;
         return bfail(e == cudaErrorMemoryAllocation ? HOUGH_ENOMEM : HOUGH_ECUDA, "hough_batch_create allocation failed");
@@ -258,18 +256,16 @@ int hough::batch_run(hough_batch *b, const float *r, const float *phi, const flo
         it = b->graphs.emplace(n_events, exec).first;
     }
     BCU(cudaGraphLaunch(it->second, s), "graph launch failed");
-    note_launches(kStageLaunches + kVoteLaunches + peak_launches(n_events) + kStage2Launches);
+    note_launches(kStageLaunches + kVoteLaunches + kPeakLaunches + kStage2Launches);
     b->n_events = n_events;
     b->ran = true;
     return HOUGH_OK;
 }
 
-// Enqueue the concatenation of the last run's candidates into the batch's device buffer and the
-// copy of the per-event offsets (int32, n_events + 1) to `offsets_host`; no synchronisation.
+// Enqueue the copy of the last run's per-event offsets (int32, n_events + 1) to `offsets_host`; no
+// synchronisation.
 int hough::batch_enqueue_offsets(hough_batch *b, int32_t *offsets_host, cudaStream_t s)
 {
-    BCU(launch_pack_candidates(b->ax, b->w, b->packed, s), "pack kernel failed");
-    note_launches(1);
     BCU(cudaMemcpyAsync(offsets_host, b->w.cand_base, sizeof(int32_t) * (b->n_events + 1), cudaMemcpyDeviceToHost, s),
         "copy offsets failed");
     return HOUGH_OK;
@@ -278,11 +274,9 @@ int hough::batch_enqueue_offsets(hough_batch *b, int32_t *offsets_host, cudaStre
 int hough::batch_enqueue_offsets_mapped(hough_batch *b, int32_t *offsets_host, hough_candidate *mapped, int64_t cap,
                                         cudaStream_t s)
 {
-    BCU(launch_pack_candidates(b->ax, b->w, mapped, s, cap, b->packed), "pack kernel failed");   // the rest stays on the device
+    BCU(launch_copy_candidates(b->w, mapped, s, cap), "copy kernel failed");   // the rest stays on the device
     note_launches(1);
-    BCU(cudaMemcpyAsync(offsets_host, b->w.cand_base, sizeof(int32_t) * (b->n_events + 1), cudaMemcpyDeviceToHost, s),
-        "copy offsets failed");
-    return HOUGH_OK;
+    return batch_enqueue_offsets(b, offsets_host, s);
 }
 
 // Enqueue the copy of the first n events' counters to `stats_host`; no synchronisation.
@@ -294,12 +288,12 @@ int hough::batch_enqueue_stats(hough_batch *b, DevStats *stats_host, int n, cuda
 
 size_t hough::batch_device_bytes(const hough_batch *b) { return b->device_bytes; }
 
-// Enqueue the copy of packed candidates [first, n) to dst_host[0, n - first); no synchronisation.
+// Enqueue the copy of candidates [first, n) to dst_host[0, n - first); no synchronisation.
 int hough::batch_enqueue_candidates(hough_batch *b, hough_candidate *dst_host, int64_t n, cudaStream_t s,
                                     int64_t first)
 {
     if (n > first)
-        BCU(cudaMemcpyAsync(dst_host, b->packed + first, sizeof(hough_candidate) * (n - first),
+        BCU(cudaMemcpyAsync(dst_host, b->w.cands + first, sizeof(hough_candidate) * (n - first),
                             cudaMemcpyDeviceToHost, s),
             "copy candidates failed");
     return HOUGH_OK;
@@ -340,7 +334,7 @@ int hough_batch_profile(hough_batch *b, const float *r, const float *phi, const 
     if (!e) e = cudaEventRecord(ev[6], s);
     if (!e) e = cudaStreamSynchronize(s);
     if (e) return done(bfail(HOUGH_ECUDA, "profiled batch run failed"));
-    note_launches(kStageLaunches + kVoteLaunches + peak_launches(n_events) + kStage2Launches);
+    note_launches(kStageLaunches + kVoteLaunches + kPeakLaunches + kStage2Launches);
     b->n_events = n_events;
     b->ran = true;
     float ms[6];
@@ -380,15 +374,9 @@ int hough_batch_candidates(hough_batch *b, hough_candidate *out, int64_t cap, in
     const int64_t total = base[E];
     const int64_t ncopy = std::min(total, cap);
     if (ncopy > 0) {
-        hough_candidate *dst = where == HOUGH_DEVICE && ncopy == total ? out : b->packed;
-        Workspace w = b->w;
-        w.n_events = E;
-        BCU(launch_pack_candidates(b->ax, w, dst, s), "pack kernel failed");
-        note_launches(1);
-        if (dst != out)
-            BCU(cudaMemcpyAsync(out, b->packed, sizeof(hough_candidate) * ncopy,
-                                where == HOUGH_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, s),
-                "copy candidates failed");
+        BCU(cudaMemcpyAsync(out, b->w.cands, sizeof(hough_candidate) * ncopy,
+                            where == HOUGH_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, s),
+            "copy candidates failed");
         BCU(cudaStreamSynchronize(s), "synchronise failed");
     }
     if (total > cap) return bfail(HOUGH_ETRUNC, "more candidates than the capacity");

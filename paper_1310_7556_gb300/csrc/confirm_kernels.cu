@@ -2,48 +2,52 @@
 // expensive computations"): for each candidate, the hits whose stage-1 vote fell in its cell
 // (membership) and their vote in a (cot theta, z0) grid of layer masks (stage 2).
 //
-// One kernel, confirm_kernel, with a group of threads per candidate: a warp in batches (thousands
-// of candidates keep every SM busy), a CTA of four warps for a single event (a few hundred
-// candidates, whose time is the chain of one candidate).  Groups stride over all events'
-// candidates, flattened.  Per candidate:
+// One kernel, confirm_kernel.  A warp takes a group of C consecutive candidates of the flattened
+// list (three for detectors of at most 10 layers, two for more; fewer when there are not enough
+// candidates to fill the GPU's warps) and goes through
 //
-//   1. Segments.  Only layers present in the candidate's mask can hold members (with the count
+//   1. Ranges.  Only layers present in a candidate's mask can hold members (with the count
 //      accumulator every layer is scanned).  For a layer whose hits share one radius the vote
 //      inverts exactly -- a hit of bucket J votes into column j on row i when
-//      J = j + I_i + (f < g_i) -- so two buckets of the (layer, azimuth bucket)-sorted hits hold
-//      all of that layer's members: bucket j + I_i with f >= g_i and bucket j + I_i + 1 with
-//      f < g_i.  Other layers give the buckets their radius range allows, whose hits redo the vote
-//      (FP32 with FP64 refinement, as in the vote kernel).  Lane t of the first warp computes
-//      range t = (layer t / 2, side t % 2); the non-empty ones are compacted with their exclusive
-//      prefix, so their starts strictly increase.
-//   2. Membership.  The group tests the flattened union of the ranges, a lane per hit.  A lane's
-//      range is found without a search: the ranges starting inside the warp's window of 32 hits
+//      J = j + I_i + (f < g_i) -- so two neighbouring buckets of the (layer, azimuth bucket)-sorted
+//      hits hold all of that layer's members: bucket j + I_i with f >= g_i and the one after it
+//      with f < g_i.  A lane per (candidate, layer) forms that one range, its split point and the
+//      jump at the split where the second bucket wraps around phi.  Other layers give the buckets
+//      their radius range allows, whose hits redo the vote (FP32 with FP64 refinement, as in the
+//      vote kernel).
+//   2. Membership.  The warp tests the flattened union of all C candidates' ranges, a lane per hit.
+//      A lane's range is found without a search: the ranges starting inside the window of 32 hits
 //      are OR-reduced into one bit mask (a redux), and a population count below the lane gives its
-//      range.  Members are ranked by ballot in the fixed order (layer, bucket, position) and
-//      listed, each with its z, in the group's shared memory.
-//   3. Coefficients.  A lane per listed member (so this arithmetic runs once per 32 members, not
-//      once per 32 hits scanned): the z0 coordinate of its vote on cot row m,
+//      range.  Members are listed by ballot in the fixed order (candidate, layer, position).
+//   3. Coefficients, a lane per listed member, 32 members a round whatever candidates they belong
+//      to: the z0 coordinate of its vote on cot row m,
 //      w(m) = n_z0 (z - s t_m - z0_min) / (z0_max - z0_min) = a - (m - m_ref) b, evaluated in FP32
 //      around the row m_ref where it crosses z0_min, from coefficients formed in two-float
-//      arithmetic (to within 2e-5 bin of its exact value), and the exact run of rows whose vote
-//      falls inside the z0 range (w is monotone in m, so they form one run).  Members with a
-//      non-empty run are compacted in place with the exclusive prefix of the run lengths.
-//   4. Stage-2 vote.  The (member, row) pairs of all runs are spread over the lanes -- a pair's
-//      member found like a hit's range above -- and voted with a shared atomicOr into the group's
-//      own n_cot x n_z0 grid (16-bit masks, or in batches of a detector of at most 10 layers
-//      10-bit masks three to a word, 5.3 KB for 64 x 64).  The word the atomic returns judges the
-//      cell: the last OR into a cell sees its final mask and every earlier one a subset, so the
-//      largest popcount seen is the grid's maximum and the lowest cell seen with it the
-//      row-major-first arg-max.  Each lane keeps the best as one 32-bit key (popcount, then the
-//      complement of the cell index), and a redux finds the group's.
-//   5. The cell's final mask is read back, the touched rows cleared, the candidate written.
+//      arithmetic (to within 2e-5 bin of its exact value), and the run of rows whose vote falls
+//      inside the z0 range (w is monotone in m, so they form one run).
+//   4. Stage-2 vote, candidate by candidate.  The (member, row) pairs of a candidate's runs are
+//      spread over the lanes -- a pair's member found by a population count of a bit array that
+//      marks each run's first pair -- and voted with a shared atomicOr into the warp's
+//      n_cot x n_z0 grid (16-bit masks, or for detectors of at most 10 layers 10-bit masks three
+//      to a word, 5.3 KB for 64 x 64).  The word the atomic returns judges the cell: the last OR
+//      into a cell sees its final mask and every earlier one a subset, so the largest popcount
+//      seen is the grid's maximum and the lowest cell seen with it the row-major-first arg-max.
+//      Each lane keeps the best as one 32-bit key (popcount, then the complement of the cell
+//      index), and a redux finds the warp's.
+//   5. The cell's final mask is read back, the grid cleared, the record written.
 //
-// A candidate with more members than the list holds (kBatchCap, kEventCap), or whose runs hold more
-// pairs than a chunk votes at a time, is done in chunks, the membership pass repeated for each,
-// all chunks voting into the one grid.  The member lists are kept for contexts (hough_get_members
-// reads them), in the event's member pool, where a slot is reserved once the membership pass has
-// counted the members and step 3 stores each member as it reads it; a batch keeps none.  The event's member and stage-2
-// vote counters are summed per group and added once per event a group visits.
+// Why groups of candidates: a candidate of a batch scans about 30 hits of 9 layers, has 15 members
+// and casts 140 stage-2 votes, so with one candidate a warp the lanes of steps 1-3 were half idle
+// and their fixed cost (prefix sums, compactions, broadcasts) was paid per candidate.  Only the
+// vote needs a grid of its own, and it alone is done a candidate at a time, so a group costs no
+// more shared memory than a candidate did.
+//
+// When the list is full its members go through steps 3 and 4 before further hits are tested, a
+// candidate's grid, best key and counts being carried on.  The member lists are kept for contexts (hough_get_members
+// reads them), in the event's member pool, where a slot is reserved once a candidate's members are
+// counted; a batch keeps none.  The event's member and stage-2 vote counters are summed per warp
+// and added once per event a warp visits.
+#include <algorithm>
 #include <atomic>
 #include <climits>
 
@@ -53,178 +57,48 @@ namespace hough {
 
 namespace {
 
-constexpr int kBatchCap = 40;      // members a warp holds at a time (batches)
-constexpr int kBatchPairs = 1024;  // (member, row) pairs a warp votes at a time (batches)
-constexpr int kEventCap = 256;     // members a four-warp group holds at a time (single events)
-constexpr int kEventPairs = 4096;  // pairs it votes at a time
-constexpr int kEventWarps = 4;     // warps per candidate for a single event
-constexpr int kBatchGroups = 4;    // one-warp groups per CTA at most (batches)
-constexpr int kMaxBandsRead = 8192;   // band offsets a single event's CTA may hold to read the band lists
-constexpr int kManyPerCta = 2;        // one event with more candidates than this per CTA: a warp per candidate
+constexpr int kWarps = 4;             // warps per CTA at most (fewer when their grids do not fit)
+constexpr int kListCap = 96;          // members a warp lists at a time
+constexpr int kMaxBandsRead = 8192;   // bands of a single event whose lists the confirmation reads itself
+constexpr int kTeamRounds = 2;        // one event with at most so many candidates per CTA: its warps share each candidate
+constexpr int kBandChunks = 64;       // coarse band offsets a CTA holds to do so
 
-// Per-group scratch of a group of WPC warps, for detectors of at most NL layers.  Kind of a range: bits 0..3 the layer, bit 4 the side (1: f < g), bit 5 a
-// layer whose hits lie at several radii (each hit's vote recomputed).
-template <int WPC, int CAP, int MAXP, int NL>
+// Per-warp scratch; the start bits of the runs and the grid follow it.
 struct __align__(16) Scratch {
-    // chunk member with a run of cot rows: a, b (float bits); (first row - first pair - m_ref) +
-    // kDmBias in bits 0..19 and the layer in bits 20..23; (first row - first pair) * n_z0
-    int4 par[CAP];
-    float4 zco[NL];                 // stage-2 terms {S hi, S lo, B hi, B lo} of each table layer at this row
-    float rb[NL];                   // 1 / B hi of each table layer at this row (approximate)
-    unsigned starts[MAXP / 32];     // bit v: a chunk member's run starts at pair v
-    int seg_pre[2 * NL], seg_start[2 * NL];   // the ranges, two a layer at most
-    unsigned seg_kind[2 * NL];
-    float seg_g[2 * NL];
-    int wtmp[4 * WPC];
-    int n_seg, total, pool_base, pool_written;
+    int4 par[32];           // a round's members with a run of cot rows: a, b, (first row - first pair - m_ref) (float bits);
+                            // (first row - first pair) * n_z0 * 32 + layer
+    float4 zco[32];         // stage-2 terms {S hi, S lo, B hi, B lo} by lane (candidate, layer)
+    int4 seg[32];           // the non-empty ranges: staged position less flattened index, flattened index of the
+                            // split, g (float bits), jump of the staged position at the split
+    int list_p[kListCap];   // the chunk's members: staged position
+    unsigned char list_slot[kListCap];   // and slot
+    unsigned char seg_slot[32];          // lane (candidate, layer) of a range, bit 5: a layer of several radii
 };
 
-constexpr int kDmBias = 1 << 19;
-
-template <int WPC>
-__device__ __forceinline__ void group_sync()
-{
-    if (WPC == 1) __syncwarp(); else __syncthreads();
-}
-
-template <int WPC>
-__device__ __forceinline__ int group_tid() { return WPC == 1 ? (int)(threadIdx.x & 31) : (int)threadIdx.x; }
-
-template <int WPC>
-__device__ __forceinline__ int group_warp() { return WPC == 1 ? 0 : (int)(threadIdx.x >> 5); }
+// What the warps of a team exchange.
+struct Team {
+    unsigned best[kWarps];
+    int members[kWarps];
+    int pool_base, pool_n;
+};
 
 __device__ __forceinline__ unsigned lanes_below() { return (1u << (threadIdx.x & 31)) - 1u; }
 
-// Rank of this thread among the group's threads with `pred` set (group order: warp, then lane);
-// *total receives their number.  Called by every thread of the group.
-template <int WPC>
-__device__ __forceinline__ int group_excl_count(bool pred, int *total, int *wtmp)
+__device__ __forceinline__ TabEntry load_tab(const TabEntry *p)
 {
-    const unsigned b = __ballot_sync(0xFFFFFFFFu, pred);
-    const int within = __popc(b & lanes_below());
-    if (WPC == 1) {
-        *total = __popc(b);
-        return within;
-    }
-    const int w = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0) wtmp[w] = __popc(b);
-    __syncthreads();
-    int pre = 0, tot = 0;
-#pragma unroll
-    for (int k = 0; k < WPC; ++k) {
-        const int t = wtmp[k];
-        pre += k < w ? t : 0;
-        tot += t;
-    }
-    __syncthreads();
-    *total = tot;
-    return pre + within;
+    const int2 v = __ldg(reinterpret_cast<const int2 *>(p));
+    return TabEntry{v.x, __int_as_float(v.y)};
 }
 
-// Exclusive prefix of v over the group; *total receives the sum.  Called by every thread of the group.
-template <int WPC>
-__device__ __forceinline__ int group_excl_scan(int v, int *total, int *wtmp)
+__device__ __forceinline__ int warp_incl_scan(int v)
 {
     const int lane = threadIdx.x & 31;
-    int incl = v;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-        const int t = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-        if (lane >= d) incl += t;
+        const int t = __shfl_up_sync(0xFFFFFFFFu, v, d);
+        if (lane >= d) v += t;
     }
-    if (WPC == 1) {
-        *total = __shfl_sync(0xFFFFFFFFu, incl, 31);
-        return incl - v;
-    }
-    const int w = threadIdx.x >> 5;
-    if (lane == 31) wtmp[w] = incl;
-    __syncthreads();
-    int pre = 0, tot = 0;
-#pragma unroll
-    for (int k = 0; k < WPC; ++k) {
-        const int t = wtmp[k];
-        pre += k < w ? t : 0;
-        tot += t;
-    }
-    __syncthreads();
-    *total = tot;
-    return pre + incl - v;
-}
-
-// Maximum (MAX) or minimum of v over the group, returned to every thread.
-template <int WPC, bool MAX>
-__device__ __forceinline__ unsigned group_reduce(unsigned v, int *wtmp)
-{
-    v = MAX ? __reduce_max_sync(0xFFFFFFFFu, v) : __reduce_min_sync(0xFFFFFFFFu, v);
-    if (WPC == 1) return v;
-    const int w = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0) wtmp[w] = (int)v;
-    __syncthreads();
-    unsigned r = (unsigned)wtmp[0];
-#pragma unroll
-    for (int k = 1; k < WPC; ++k) r = MAX ? max(r, (unsigned)wtmp[k]) : min(r, (unsigned)wtmp[k]);
-    __syncthreads();
-    return r;
-}
-
-// Warp totals v of N quantities made group-wide: the sums over the warps before this one (pre)
-// and over all (tot), in one exchange through shared memory (wx: WPC * N words).
-template <int WPC, int N>
-__device__ __forceinline__ void group_exchange(const int (&v)[N], int (&pre)[N], int (&tot)[N], int *wx)
-{
-#pragma unroll
-    for (int n = 0; n < N; ++n) {
-        pre[n] = 0;
-        tot[n] = v[n];
-    }
-    if (WPC == 1) return;
-    const int w = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-        for (int n = 0; n < N; ++n) wx[w * N + n] = v[n];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int n = 0; n < N; ++n) {
-        int p = 0, t = 0;
-#pragma unroll
-        for (int k = 0; k < WPC; ++k) {
-            const int x = wx[k * N + n];
-            p += k < w ? x : 0;
-            t += x;
-        }
-        pre[n] = p;
-        tot[n] = t;
-    }
-    __syncthreads();
-}
-
-// Sum of v over the group, returned to every thread.
-template <int WPC>
-__device__ __forceinline__ unsigned group_reduce_add(unsigned v, int *wtmp)
-{
-    v = __reduce_add_sync(0xFFFFFFFFu, v);
-    if (WPC == 1) return v;
-    const int w = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0) wtmp[w] = (int)v;
-    __syncthreads();
-    unsigned r = 0u;
-#pragma unroll
-    for (int k = 0; k < WPC; ++k) r += (unsigned)wtmp[k];
-    __syncthreads();
-    return r;
-}
-
-// The index, within a sorted list of strictly increasing starts held one per lane (lane t: entry
-// base_idx + t, INT_MAX past the end), of the entry owning position pos0 + lane, given that entry
-// q_base owns pos0.  The entries starting inside the window (pos0, pos0 + 32) are OR-reduced into
-// a bit mask; the count of those at or below the lane's position is its offset from q_base.
-__device__ __forceinline__ int window_owner(int st_next, int pos0, int q_base)
-{
-    const int d = st_next - pos0;   // st_next: start of entry q_base + 1 + lane (no overflow: pos0 >= 0)
-    const unsigned bits = __reduce_or_sync(0xFFFFFFFFu, (d > 0 && d < 32) ? 1u << d : 0u);
-    const int lane = threadIdx.x & 31;
-    return q_base + __popc(bits & ((2u << lane) - 1u));
+    return v;
 }
 
 // The (up to two) ranges of staged hits of a layer whose hits lie at several radii that can hold
@@ -294,8 +168,8 @@ __device__ __forceinline__ bool general_member(const Axes &ax, const Workspace &
 // from the table and w(m_ref) = zscale (z - z0_min) - S - m_ref B is formed in two-float
 // arithmetic (about 2^-44 relative before the final rounding), which keeps a within a few 1e-6
 // bins of the exact value.
-__device__ __forceinline__ void table_coefficients(const Axes &ax, const float4 zc, float rb, float z, int l,
-                                                   float *a_out, float *b_out, int *mrl_out)
+__device__ __forceinline__ void table_coefficients(const Axes &ax, const float4 zc, float rb, float z, float *a_out,
+                                                   float *b_out, float *mref_out)
 {
     // d = z - z0_min and Z = zscale d as two-float values
     float2 d = two_sum(z, -ax.zmin_hi);
@@ -306,19 +180,18 @@ __device__ __forceinline__ void table_coefficients(const Axes &ax, const float4 
     float2 A = two_sum(zp.x, -zc.x);
     A.y = A.y + (zlo - zc.y);
     // any nearby row will do
-    const int mref = zc.z > 0.f ? (int)fminf(fmaxf(rintf(A.x * rb), 0.f), (float)(ax.n_cot - 1)) : 0;
+    const float fm = zc.z > 0.f ? fminf(fmaxf(rintf(A.x * rb), 0.f), (float)(ax.n_cot - 1)) : 0.f;
     // a = A - m_ref B; m_ref B.hi is exact as a two-float product
-    const float fm = (float)mref;
     const float2 q = two_prod(fm, zc.z);
     *a_out = __fsub_rn(A.x, q.x) + (A.y - q.y - fm * zc.w);
     *b_out = zc.z;
-    *mrl_out = mref | (l << 16);
+    *mref_out = fm;
 }
 
 // The same for a member of a layer whose hits lie at several radii: the arc length from the
 // closest approach in FP64 (r asin(|x|) / |x| for prompt tracks).
-__device__ __forceinline__ void exact_coefficients(const Axes &ax, int l, int i, const ColdHit &ch, float *a_out,
-                                                   float *b_out, int *mrl_out)
+__device__ __forceinline__ void exact_coefficients(const Axes &ax, int i, const ColdHit &ch, float *a_out,
+                                                   float *b_out, float *mref_out)
 {
     const double rd = (double)ch.r;
     const double x = __dmul_rn(sagitta_coef(ax, rd), qpt_centre(ax, i));
@@ -329,22 +202,11 @@ __device__ __forceinline__ void exact_coefficients(const Axes &ax, int l, int i,
     const double t0 = __dadd_rn(ax.cot_min, __dmul_rn(0.5, ax.dt));
     const double A = __dmul_rn(ax.zscale, __dsub_rn(__dsub_rn((double)ch.z, ax.z0_min), __dmul_rn(s, t0)));
     const double B = __dmul_rn(ax.zscale, __dmul_rn(s, ax.dt));
-    int mref = 0;
-    if (B > 0.0) mref = (int)fminf(fmaxf(rintf((float)A / (float)B), 0.f), (float)(ax.n_cot - 1));
+    float mref = 0.f;
+    if (B > 0.0) mref = fminf(fmaxf(rintf((float)A / (float)B), 0.f), (float)(ax.n_cot - 1));
     *a_out = (float)(A - (double)mref * B);
     *b_out = (float)B;
-    *mrl_out = mref | (l << 16);
-}
-
-// z0 bin of a member's vote at cot row m, -1 outside the grid: w(m) = a - (m - m_ref) b in FP32,
-// one fused multiply-add from the two-float coefficients.  Its error stays below 2e-5 bin (a to
-// ~4e-6, the rounding of b times |m - m_ref| <= 128 / b rows to ~8e-6, the final rounding to
-// ~4e-6), so every vote farther than that from a z0 edge -- in particular every vote the exact
-// definition would not flag within 1e-4 bin -- lands in the bin the definition gives.
-__device__ __forceinline__ int stage2_cell(const Axes &ax, float a, float b, int mrl, int m)
-{
-    const float wv = fmaf(-(float)(m - (mrl & 0xFFFF)), b, a);
-    return (wv >= 0.f && wv < (float)ax.n_z0) ? (int)wv : -1;   // truncation is the floor here
+    *mref_out = mref;
 }
 
 // The run of cot rows whose vote of the member can fall inside the z0 range.  w(m) is the rounding
@@ -352,41 +214,24 @@ __device__ __forceinline__ int stage2_cell(const Axes &ax, float a, float b, int
 // 0 <= w(m) < n_z0 form one run.  Approximate quotients bound the run from outside by about a row
 // on each side; one step at each end then drops a bound whose own vote falls outside, which
 // leaves the exact run in all but rare cases (a row of an outer bound still outside: every pair
-// is tested again when it votes).  *len receives the length (0: no row).
-__device__ __forceinline__ void member_run(const Axes &ax, float a, float b, float rb, int mrl, int *lo_out,
+// is tested again when it votes).  Rows are whole numbers held as floats (at most 256, exact).
+// *len receives the length (0: no row).
+__device__ __forceinline__ void member_run(float n_cot, float n_z0, float a, float b, float rb, float mref, float *lo_out,
                                            int *len_out)
 {
-    const int mref = mrl & 0xFFFF;
-    const float top = (float)(ax.n_cot - 1);
-    const float flo = floorf((float)mref + (a - (float)ax.n_z0) * rb);   // rb: about 1 / b
-    const float fhi = floorf((float)mref + a * rb) + 1.f;
-    int lo = (int)fminf(fmaxf(flo, 0.f), top + 1.f);
-    int hi = (int)fminf(fmaxf(fhi, -1.f), top);
-    lo += (lo <= hi && stage2_cell(ax, a, b, mrl, lo) < 0) ? 1 : 0;
-    hi -= (hi >= lo && stage2_cell(ax, a, b, mrl, hi) < 0) ? 1 : 0;
+    const float top = n_cot - 1.f;
+    const float alo = a - n_z0;
+    float lo = fminf(fmaxf(floorf(fmaf(alo, rb, mref)), 0.f), n_cot);   // rb: about 1 / b
+    float hi = fminf(fmaxf(floorf(fmaf(a, rb, mref)) + 1.f, -1.f), top);
+    const float wlo = fmaf(-(lo - mref), b, a), whi = fmaf(-(hi - mref), b, a);
+    if (!(wlo >= 0.f && wlo < n_z0)) lo += 1.f;   // (of an empty run too: it stays empty)
+    if (!(whi >= 0.f && whi < n_z0)) hi -= 1.f;
     if (!(b > 0.f)) {   // w constant in m: every row or none
-        const bool in = a >= 0.f && a < (float)ax.n_z0;
-        lo = 0;
-        hi = in ? ax.n_cot - 1 : -1;
+        lo = 0.f;
+        hi = a >= 0.f && a < n_z0 ? top : -1.f;
     }
     *lo_out = lo;
-    *len_out = max(0, hi - lo + 1);
-}
-
-// One stage-2 vote (when `in`): OR the member's layer bit into `cell` = m n_z0 + nz of `grid`; returns
-// the key of the cell as the OR left it (0 when not `in`): its popcount above the complement of the cell index, so that the larger
-// key is the larger popcount and, on a tie, the lower cell.  P10: the grid packs three 10-bit
-// masks a word (detectors of at most 10 layers), else two 16-bit ones.
-template <bool P10>
-__device__ __forceinline__ unsigned stage2_vote(uint32_t *grid, unsigned cell, int layer, bool in)
-{
-    const unsigned word = P10 ? cell / 3u : cell >> 1;
-    const unsigned shift = P10 ? (cell - word * 3u) * 10u : (cell & 1u) << 4;
-    const uint32_t bit = 1u << layer;
-    uint32_t old = 0u;
-    if (in) old = atomicOr(&grid[word], bit << shift);
-    const uint32_t msk = ((old >> shift) & (P10 ? 0x3FFu : 0xFFFFu)) | bit;
-    return in ? ((unsigned)__popc(msk) << 16) | (0xFFFFu - cell) : 0u;
+    *len_out = (int)fmaxf(hi - lo + 1.f, 0.f);
 }
 
 template <bool P10>
@@ -397,20 +242,6 @@ __device__ __forceinline__ uint32_t grid_mask(const uint32_t *grid, unsigned cel
     return (grid[word] >> shift) & (P10 ? 0x3FFu : 0xFFFFu);
 }
 
-// Zero the grid words of rows [rlo, rhi] (16-byte stores over a span rounded out to whole vectors:
-// the extra words hold only cells outside the touched rows, already zero).
-template <int WPC, bool P10>
-__device__ __forceinline__ void clear_rows(const Axes &ax, uint32_t *grid, int rlo, int rhi)
-{
-    if (rlo > rhi) return;
-    const int c0 = rlo * ax.n_z0, c1 = (rhi + 1) * ax.n_z0 - 1;   // first and last cell
-    const int w0 = (P10 ? c0 / 3 : c0 >> 1) & ~3;
-    const int w1 = ((P10 ? c1 / 3 : c1 >> 1) | 3) + 1;   // <= grid words (a multiple of 4)
-    uint4 *g4 = reinterpret_cast<uint4 *>(grid);
-#pragma unroll 4
-    for (int q = (w0 >> 2) + group_tid<WPC>(); q < (w1 >> 2); q += 32 * WPC) g4[q] = make_uint4(0u, 0u, 0u, 0u);
-}
-
 // A candidate record as two 16-byte vectors (the arrays are 16-byte aligned, 32 bytes an entry).
 __device__ __forceinline__ void store_candidate(hough_candidate *p, const hough_candidate &c)
 {
@@ -418,466 +249,506 @@ __device__ __forceinline__ void store_candidate(hough_candidate *p, const hough_
     reinterpret_cast<uint4 *>(p)[1] = make_uint4(c.icot, c.jz0, c.mask2, c.flags);
 }
 
-// Step 2: one pass over the candidate's ranges, a lane per hit, software-pipelined (the next
-// round's hit is requested before this round is tested).  Members are ranked in the fixed order
-// (layer, bucket, position) and sink(r, p, kd, z) receives member r: its staged position, the kind
-// of its range and (Z) its z.  Returns the number of members.
-template <int WPC, int CAP, int MAXP, int NL, bool GEN, bool Z, typename Sink>
-__device__ int scan_members(const Axes &ax, const Workspace &w, Scratch<WPC, CAP, MAXP, NL> &S, const HotHit *hot,
-                            const float *fsort, const float *zsort, const ColdHit *cold, int i, int j, float s32,
-                            float refine_eps, Sink &&sink)
-{
-    const int lane = threadIdx.x & 31;
-    const int T = S.total, nseg = S.n_seg;
-    const int pre_t = lane < nseg ? S.seg_pre[lane] : INT_MAX;
-    const int start_t = lane < nseg ? S.seg_start[lane] : 0;
-    const unsigned kind_t = lane < nseg ? S.seg_kind[lane] : 0u;
-    const float g_t = lane < nseg ? S.seg_g[lane] : 0.f;
-    // the hit at flattened index base + lane: its staged position, range kind and threshold
-    auto locate = [&](int base, int &p, unsigned &kd, float &gg) {
-        const int qb = __popc(__ballot_sync(0xFFFFFFFFu, pre_t <= base)) - 1;   // range 0 starts at 0 <= base
-        const int src = qb + 1 + lane;   // the range after qb that this lane inspects
-        const int pn = __shfl_sync(0xFFFFFFFFu, pre_t, src & 31);
-        const int sg = min(window_owner(src < 32 ? pn : INT_MAX, base, qb), 31);
-        p = __shfl_sync(0xFFFFFFFFu, start_t, sg) + (base + lane - __shfl_sync(0xFFFFFFFFu, pre_t, sg));
-        kd = __shfl_sync(0xFFFFFFFFu, kind_t, sg);
-        gg = __shfl_sync(0xFFFFFFFFu, g_t, sg);
-    };
-    const int G = 32 * WPC;
-    const int wb = 32 * group_warp<WPC>();
-    int n = 0;
-    int p = 0;
-    unsigned kd = 0u;
-    float gg = 0.f, f = 0.f, z = 0.f;
-    if (wb < T) {
-        locate(wb, p, kd, gg);
-        if (wb + lane < T && !(kd & 32u)) {
-            f = __ldg(&fsort[p]);
-            if (Z) z = __ldg(&zsort[p]);
-        }
-    }
-    for (int b0 = 0; b0 < T; b0 += G) {
-        const int v = b0 + wb + lane;
-        const int bn = b0 + G + wb;
-        int pn = 0;
-        unsigned kdn = 0u;
-        float ggn = 0.f, fn = 0.f, zn = 0.f;
-        if (bn < T) {
-            locate(bn, pn, kdn, ggn);
-            if (bn + lane < T && !(kdn & 32u)) {
-                fn = __ldg(&fsort[pn]);
-                if (Z) zn = __ldg(&zsort[pn]);
-            }
-        }
-        bool mem = v < T && (f < gg) == ((kd & 16u) != 0u);   // side 1: f < g; side 0: f >= g
-        if (GEN && v < T && (kd & 32u)) mem = general_member(ax, w, hot, cold, p, i, j, s32, refine_eps);
-        int nm;
-        const int r = n + group_excl_count<WPC>(mem, &nm, S.wtmp);
-        if (mem) sink(r, p, kd, z);
-        n += nm;
-        p = pn;
-        kd = kdn;
-        gg = ggn;
-        f = fn;
-        z = zn;
-    }
-    return n;
-}
 
-// Totals of a chunk's runs.
-struct ChunkOut {
-    int npairs;     // (member, row) pairs of the members kept
-    int consumed;   // members of the list the chunk has dealt with (kept, or without a run)
+// A candidate as the confirmation takes it: (row << 16 | column), mask, event, the event's first hit.
+struct ListEntry {
+    unsigned ij, mask;
+    int e, hstart;
 };
 
-// Step 3 for the chunk's m members listed in par as {position, kind, z bits}: each one's stage-2
-// coefficients and run of cot rows, a lane per member.  The members with a run are kept, in order,
-// while their pairs fit MAXP: par is rewritten in place from slot 0 (a slot never lies past the
-// entry it comes from, and a round's entries are all read before any is written), and the bit of
-// each kept member's first pair is set in starts.  rlo / rhi widen to the rows the runs cover.
-// pool (contexts): the member list, whose first `written` ranks are stored as the entries are read.
-template <int WPC, int CAP, int MAXP, int NL, bool GEN, bool KEEP>
-__device__ ChunkOut chunk_runs(const Axes &ax, Scratch<WPC, CAP, MAXP, NL> &S, const ColdHit *cold, int i, int m, int &rlo,
-                               int &rhi, int32_t *pool, int rank0, int written)
-{
-    const int tid = group_tid<WPC>();
-    const int G = 32 * WPC;
-    for (int q = tid; q < MAXP / 32; q += G) S.starts[q] = 0u;
-    int pairs = 0, kept = 0, consumed = 0;
-    for (int b0 = 0; b0 < m; b0 += G) {
-        const int idx = b0 + tid;
-        const bool valid = idx < m;
-        int4 e = make_int4(0, 0, 0, 0);
-        if (valid) e = S.par[idx];
-        // a context lists the member (rank rank0 + idx, its staged position) in its pool slot; a
-        // member a later chunk lists again writes the same value
-        if (KEEP && valid && rank0 + idx < written) pool[rank0 + idx] = e.x;
-        group_sync<WPC>();   // the round's entries are read (and starts cleared) before any write
-        // every lane forms coefficients (a lane past the list from entry 0's zeros) and the run is
-        // dropped where not valid: no divergent branch on the table path
-        float a, bb;
-        int mrl, mlo, len;
-        const unsigned kd = (unsigned)e.y;
-        const int l = (int)(kd & 15u);
-        float rb = S.rb[l];
-        table_coefficients(ax, S.zco[l], rb, __int_as_float(e.z), l, &a, &bb, &mrl);
-        if (GEN && valid && (kd & 32u)) {
-            exact_coefficients(ax, l, i, cold[e.x], &a, &bb, &mrl);
-            rb = bb > 0.f ? __frcp_rn(bb) : 0.f;
-        }
-        member_run(ax, a, bb, rb, mrl, &mlo, &len);
-        if (!valid) len = 0;
-        // pair prefix over the round (members without a run add nothing); a member whose pairs end
-        // past MAXP, and every one after it (their prefixes only grow), waits for the next chunk
-        int tot_len;
-        const int st = pairs + group_excl_scan<WPC>(len, &tot_len, S.wtmp);
-        const bool after = valid && st + len > MAXP;
-        const bool keep = len > 0 && !after;
-        const unsigned bkeep = __ballot_sync(0xFFFFFFFFu, keep);
-        int pre[3], tot[3];
-        group_exchange<WPC, 3>({__popc(bkeep), (int)__reduce_add_sync(0xFFFFFFFFu, keep ? (unsigned)len : 0u),
-                                __popc(__ballot_sync(0xFFFFFFFFu, after))},
-                               pre, tot, S.wtmp);
-        if (WPC == 1) __syncwarp();
-        if (keep) {
-            const int slot = kept + pre[0] + __popc(bkeep & lanes_below());
-            const int c0 = mlo - st;
-            S.par[slot] = make_int4(__float_as_int(a), __float_as_int(bb),
-                                    (c0 - (mrl & 0xFFFF) + kDmBias) | ((mrl >> 16) << 20), c0 * ax.n_z0);
-            atomicOr(&S.starts[st >> 5], 1u << (st & 31));
-            rlo = min(rlo, mlo);
-            rhi = max(rhi, mlo + len - 1);
-        }
-        kept += tot[0];
-        pairs += tot[1];
-        consumed += min(G, m - b0) - tot[2];
-        if (tot[2] > 0) break;
-    }
-    return {pairs, consumed};
-}
-
-// Stage-2 vote of the chunk's pairs (step 4); best keeps the lane's largest key and votes its
-// count of votes cast.  Each warp takes windows of 32 consecutive pairs, one word of the start bits:
-// the member owning pair bw + lane is the number of runs starting at or before it, less one -- the
-// runs starting before the window (counted as the windows go by) plus a population count of the
-// window's bits up to the lane.  A lane's owner is a kept member past npairs too (pair 0 starts a
-// run), so every lane reads a valid entry and only the atomic is predicated.
-template <int WPC, int CAP, int MAXP, int NL, bool P10>
-__device__ void vote_pairs(const Axes &ax, const Scratch<WPC, CAP, MAXP, NL> &S, uint32_t *grid, int npairs,
-                           unsigned &best, unsigned &votes)
-{
-    const int lane = threadIdx.x & 31;
-    const unsigned upto = (2u << lane) - 1u;
-    const float nz0 = (float)ax.n_z0;
-    const int wg = group_warp<WPC>();
-    auto vote = [&](int v, int owner) {
-        const int4 pr = S.par[owner];
-        // w(m) = a - (m - m_ref) b at the pair's row m, as stage2_cell evaluates it
-        const float wv = fmaf(-(float)(v + (pr.z & 0xFFFFF) - kDmBias), __int_as_float(pr.y), __int_as_float(pr.x));
-        const bool in = v < npairs && wv >= 0.f && wv < nz0;
-        best = max(best, stage2_vote<P10>(grid, (unsigned)(v * ax.n_z0 + pr.w + (int)wv), pr.z >> 20, in));
-        votes += in ? 1u : 0u;
-    };
-    int before = 0;   // runs starting in the windows before this warp's current one
-    if constexpr (WPC == 1) {
-        // two windows an iteration: two independent chains for the scheduler to interleave
-        for (int bw = 0; bw < npairs; bw += 64) {
-            const int q = bw >> 5;
-            const unsigned b0 = S.starts[q], b1 = q + 1 < MAXP / 32 ? S.starts[q + 1] : 0u;
-            const int n0 = __popc(b0);
-            vote(bw + lane, before + __popc(b0 & upto) - 1);
-            if (bw + 32 < npairs) vote(bw + 32 + lane, before + n0 + __popc(b1 & upto) - 1);   // (warp-uniform)
-            before += n0 + __popc(b1);
-        }
-    } else {
-        for (int k = 0; k < wg; ++k) before += __popc(S.starts[k]);
-        for (int bw = 32 * wg; bw < npairs; bw += 32 * WPC) {
-            const unsigned bits = S.starts[bw >> 5];
-            const int owner = before + __popc(bits & upto) - 1;
-#pragma unroll
-            for (int k = 0; k < WPC; ++k)
-                if ((bw >> 5) + k < MAXP / 32) before += __popc(S.starts[(bw >> 5) + k]);
-            vote(bw + lane, owner);
-        }
-    }
-}
-
-// Exclusive prefix of counts[0, n) into out[0, n] (out[n]: the sum, also returned), by the whole CTA.
-__device__ int block_excl_scan(const int32_t *counts, int n, int *out)
+// One event whose list was not compacted: the CTA scans the band counts, keeping the offset of the
+// first band of each of kBandChunks chunks of `chunk` bands in `coarse` (coarse[kBandChunks]: the
+// total).  A candidate's band is then found by a search over the coarse offsets and a walk over the
+// counts of one chunk.
+__device__ int scan_bands(const int32_t *counts, int nb, int chunk, int *coarse)
 {
     __shared__ int s_w[32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    const int chunk = (n + blockDim.x - 1) / blockDim.x;
-    const int k0 = min(n, (int)threadIdx.x * chunk), k1 = min(n, k0 + chunk);
-    int sum = 0;
-    for (int k = k0; k < k1; ++k) sum += counts[k];
-    int incl = sum;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const int t = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-        if (lane >= d) incl += t;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    int carry = 0;
+    for (int c0 = 0; c0 < kBandChunks; c0 += blockDim.x) {
+        const int c = c0 + threadIdx.x;
+        const int k0 = min(nb, c * chunk), k1 = min(nb, k0 + chunk);
+        int sum = 0;
+        for (int k = k0; k < k1; ++k) sum += counts[k];
+        const int incl = warp_incl_scan(sum);
+        __syncthreads();
+        if (lane == 31) s_w[warp] = incl;
+        __syncthreads();
+        int before = carry, all = 0;
+        for (int k = 0; k < nw; ++k) {
+            before += k < warp ? s_w[k] : 0;
+            all += s_w[k];
+        }
+        if (c < kBandChunks) coarse[c] = before + incl - sum;
+        carry += all;
     }
-    if (lane == 31) s_w[warp] = incl;
+    if (threadIdx.x == 0) coarse[kBandChunks] = carry;
     __syncthreads();
-    int before = 0, all = 0;
-    for (int k = 0; k < nw; ++k) {
-        before += k < warp ? s_w[k] : 0;
-        all += s_w[k];
-    }
-    int run = before + incl - sum;
-    for (int k = k0; k < k1; ++k) {
-        out[k] = run;
-        run += counts[k];
-    }
-    if (threadIdx.x == 0) out[n] = all;
-    __syncthreads();
-    return all;
+    return carry;
 }
 
-// Membership and stage 2 of every candidate a group takes.  GEN: some layer's hits lie at several
-// radii (their votes are redone per hit, partly in FP64); without it that code is left out, which
-// spares the common path its registers.  KEEP: the member lists may be kept (Workspace::keep_members
-// decides; single events only), code the batches' one-warp kernels leave out for the same reason.
-template <int WPC, int CAP, int MAXP, int NL, bool P10, bool GEN, bool KEEP>
-__device__ __forceinline__ void confirm_all(const Axes &ax, const Workspace &w, float s32, float refine_eps,
-                                            Scratch<WPC, CAP, MAXP, NL> &S, uint32_t *grid, const LayerInfo *s_info,
-                                            int ngroups, int gidx, int total, const int *band_offs)
+// Membership and stage 2 of every group of C candidates the warp takes.  NL: layers a candidate has
+// lanes for.  GEN: some layer's hits lie at several radii (their votes are redone per hit, partly in
+// FP64); without it that code is left out, which spares the common path its registers.
+// G64: the stage-2 grid is 64 x 64 (its sizes are then constants of the code).
+// TEAM: the CTA's kWarps warps share one candidate at a time (C is 1): each takes every kWarps-th
+// window of its hits through steps 2-4 with a list of its own, voting into one grid, and they meet
+// to combine their keys.  KEEP: the member lists are kept.
+template <int NL, bool P10, bool G64, bool GEN, bool KEEP, bool TEAM>
+__device__ __forceinline__ void confirm_groups(const Axes &ax, const Workspace &w, float s32, float refine_eps,
+                                               Scratch &S, Team *team, unsigned *starts, uint32_t *grid, const int grid_vecs,
+                                               unsigned layers_present, unsigned layers_general, int C, int first, int step,
+                                               int total, const int *coarse, int chunk)
 {
-    const int tid = group_tid<WPC>(), lane = threadIdx.x & 31, wg = group_warp<WPC>();
-    const int L = ax.n_layers, nphi = ax.n_phi, nkeys = L * nphi;
-    // the event's counters, summed by the group's first thread over the event's candidates it takes
-    int acc_e = -1;
-    unsigned acc_members = 0u;
-    unsigned long long acc_votes = 0ull;
-    // candidate f goes to CTA f mod gridDim, so that a few candidates spread over all SMs; a group's
-    // candidates come in increasing flattened order, so its event only moves forward
-    int e = 0, e_base = 0, e_next = w.n_events == 1 ? INT_MAX : -1;   // the event of the last candidate fetched
-    // (i, j, mask) of candidate f, whose event becomes e; the next candidate's is requested while
-    // this one is confirmed, taking its loads off the candidate's chain
-    auto fetch = [&](int f) {
-        if (e_next < 0) {
-            e = upper_index(w.cand_base, w.n_events, f);
-            e_base = w.cand_base[e];
-            e_next = w.cand_base[e + 1];
+    const int lane = threadIdx.x & 31;
+    constexpr int TW = TEAM ? kWarps : 1;
+    const int wpos = TEAM ? (int)(threadIdx.x >> 5) : 0;
+    const unsigned upto = (2u << lane) - 1u;
+    const int nphi = ax.n_phi, nkeys = ax.n_layers * nphi;
+    const int kc = lane / NL, l = lane - kc * NL;   // the lane's candidate of the group and layer
+    const bool lane_on = kc < C && l < ax.n_layers;
+    const int n_z0 = G64 ? 64 : ax.n_z0;
+    const float n_z0f = (float)n_z0, n_cotf = G64 ? 64.f : (float)ax.n_cot;
+    const unsigned grid_s = smem_u32(grid);
+    // the event's counters, summed over the candidates of one event and added when it changes (a
+    // lane's own votes are added up over the warp only then)
+    int acc_e = 0;
+    unsigned acc_members = 0u, acc_votes = 0u;
+    auto flush = [&](int e) {
+        const unsigned long long v = (unsigned long long)__reduce_add_sync(0xFFFFFFFFu, acc_votes & 0xFFFFu) +
+                                     ((unsigned long long)__reduce_add_sync(0xFFFFFFFFu, acc_votes >> 16) << 16);
+        if (lane == 0) {
+            if (acc_members) atomicAdd(&w.stats[acc_e].n_members, acc_members);
+            if (v) atomicAdd(&w.stats[acc_e].stage2_votes, v);
         }
-        while (f >= e_next) {
-            ++e;
-            e_base = e_next;
-            e_next = w.cand_base[e + 1];
-        }
-        const int c = f - e_base;
-        if (band_offs) {
-            // one event whose candidate list was not compacted: candidate c from its band's list
-            int b = 0, hi = n_bands(ax, w.band_rows) - 1;   // the last band with offset <= c (shared memory)
-            while (b < hi) {
-                const int mid = (b + hi + 1) >> 1;
-                if (band_offs[mid] <= c) b = mid; else hi = mid - 1;
-            }
-            const uint2 v = w.band_cands[(int64_t)b * w.band_cap + (c - band_offs[b])];
-            return make_uint3(v.x / (unsigned)nphi, v.x % (unsigned)nphi, v.y);
-        }
-        const uint4 v = *reinterpret_cast<const uint4 *>(w.cands + (int64_t)e * w.max_cand + c);
-        return make_uint3(v.x, v.y, v.z);
+        acc_e = e;
+        acc_members = acc_votes = 0u;
     };
-    const int stride = gridDim.x * ngroups;
-    int f = gidx * gridDim.x + blockIdx.x;
-    uint3 rec = f < total ? fetch(f) : make_uint3(0u, 0u, 0u);
-    for (; f < total; f += stride) {
-        const int ev = e, c = f - e_base;
-        hough_candidate cd;
-        cd.iq = rec.x;
-        cd.jphi = rec.y;
-        cd.mask = rec.z;
-        cd.n_members = cd.icot = cd.jz0 = cd.mask2 = cd.flags = 0u;
-        if (f + stride < total) rec = fetch(f + stride);
-        const int64_t hstart = ev == 0 ? 0 : w.hit_start[ev];   // hit_start[0] is 0
-        const HotHit *hot = w.hot + hstart;
-        const float *fsort = w.fsort + hstart;
-        const float *zsort = w.zsort + hstart;
-        const ColdHit *cold = w.cold + hstart;
-        const int32_t *offs = w.offs + (int64_t)ev * (nkeys + 1);
-        hough_candidate *cands = w.cands + (int64_t)ev * w.max_cand;
-        const int i = (int)cd.iq, j = (int)cd.jphi;
-        // step 1: the candidate's ranges, lane t of the first warp taking range t = (layer t/2, side t%2)
-        if (wg == 0) {
-            const int l = lane >> 1, side = lane & 1;
-            const uint32_t mask = ax.counts ? 0xFFFFu : cd.mask;   // a count names no layers
-            int st = 0, len = 0;
-            unsigned kind = 0u;
-            float gv = 0.f;
-            if (l < L && ((mask >> l) & 1u)) {
-                const LayerInfo li = s_info[l];
-                if (li.present && li.uniform) {
-                    if (i >= li.lo && i <= li.hi) {
-                        const TabEntry te = w.tab[l * ax.n_qpt + i];
-                        const float4 zc = w.zco[l * ax.n_qpt + i];
-                        if (te.I != kNoVote) {
-                            const int J = wrap_col(j + te.I + side, nphi);   // |I| <= nphi / 4 + 1
-                            st = offs[l * nphi + J];
-                            len = offs[l * nphi + J + 1] - st;
-                            kind = (unsigned)l | ((unsigned)side << 4);
-                            gv = te.g;
-                            if (side == 0) {
-                                S.zco[l] = zc;
-                                S.rb[l] = zc.z > 0.f ? __fdividef(1.f, zc.z) : 0.f;   // approximate suffices
-                            }
-                        }
-                    }
-                } else if (GEN && li.present) {
-                    int sts[2] = {0, 0}, ens[2] = {0, 0};
-                    const int nr = general_ranges(ax, w, offs, l, i, j, s32, sts, ens);
-                    if (side < nr) {
-                        st = sts[side];
-                        len = ens[side] - sts[side];
-                        kind = (unsigned)l | ((unsigned)side << 4) | 32u;
-                    }
-                }
-            }
-            int incl = len;
+
+    auto fetch = [&](int f0) {
+        ListEntry r{0u, 0u, 0, 0};
+        const int f = f0 + kc;
+        if (kc >= C || f >= total) return r;
+        if (!coarse) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(w.cand_list) + f);
+            r.ij = v.x;
+            r.mask = v.y;
+            r.e = (int)v.z;
+            r.hstart = (int)v.w;
+            return r;
+        }
+        int b = 0;   // the last chunk of bands starting at or before f
 #pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const int t = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-                if (lane >= d) incl += t;
-            }
-            const unsigned ne = __ballot_sync(0xFFFFFFFFu, len > 0);
-            if (len > 0) {
-                const int ct = __popc(ne & lanes_below());
-                S.seg_pre[ct] = incl - len;
-                S.seg_start[ct] = st;
-                S.seg_kind[ct] = kind;
-                S.seg_g[ct] = gv;
-            }
-            if (lane == 31) {
-                S.n_seg = __popc(ne);
-                S.total = incl;
+        for (int d = kBandChunks / 2; d > 0; d >>= 1)
+            if (coarse[b + d] <= f) b += d;
+        int rem = f - coarse[b];
+        for (b *= chunk;; b += 4) {   // four counts at a time; the walk ends inside the chunk
+            int c[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) c[q] = b + q < w.n_band_lists ? __ldg(&w.band_counts[b + q]) : INT_MAX;
+            if (rem < c[0]) break;
+            rem -= c[0];
+            if (rem < c[1]) { b += 1; break; }
+            rem -= c[1];
+            if (rem < c[2]) { b += 2; break; }
+            rem -= c[2];
+            if (rem < c[3]) { b += 3; break; }
+            rem -= c[3];
+        }
+        const uint2 v = __ldg(&w.band_cands[(int64_t)b * w.band_cap + rem]);
+        r.ij = v.x;
+        r.mask = v.y;
+        return r;
+    };
+
+    ListEntry next = fetch(first * C);
+    for (int gq = first; gq * C < total; gq += step) {
+        const int f0 = gq * C;
+        const ListEntry rec = next;
+        if ((gq + step) * C < total) next = fetch((gq + step) * C);
+        // step 1: the range of the lane's (candidate, layer)
+        const int i = (int)(rec.ij >> 16), j = (int)(rec.ij & 0xFFFFu);
+        int st = 0, n0 = 0, len = 0, jump = 0;
+        unsigned slot = (unsigned)lane;
+        float g = 0.f;
+        float4 zc = make_float4(0.f, 0.f, 0.f, 0.f);
+        // (a count names no layers)
+        if (lane_on && (((ax.counts && f0 + kc < total ? 0xFFFFu : rec.mask) & layers_present) >> l & 1u)) {
+            const int32_t *offs = w.offs + (int64_t)rec.e * (nkeys + 1) + l * nphi;
+            if (!GEN || !((layers_general >> l) & 1u)) {
+                const TabEntry te = load_tab(&w.tab[l * ax.n_qpt + i]);
+                zc = __ldg(&w.zco[l * ax.n_qpt + i]);
+                if (te.I != kNoVote) {
+                    const int J = wrap_col(j + te.I, nphi);   // |I| <= nphi / 4 + 1
+                    const bool last = J + 1 == nphi;          // the second bucket is the layer's first
+                    const int o0 = __ldg(&offs[J]), o1 = __ldg(&offs[J + 1]);
+                    const int p0 = last ? __ldg(&offs[0]) : o1, p1 = __ldg(&offs[last ? 1 : J + 2]);
+                    st = rec.hstart + o0;
+                    n0 = o1 - o0;
+                    len = n0 + (p1 - p0);
+                    jump = p0 - o1;
+                    g = te.g;
+                }
+            } else {
+                int sts[2] = {0, 0}, ens[2] = {0, 0};
+                const int nr = general_ranges(ax, w, w.offs + (int64_t)rec.e * (nkeys + 1), l, i, j, s32, sts, ens);
+                st = rec.hstart + sts[0];
+                n0 = ens[0] - sts[0];
+                len = n0;
+                if (nr > 1) {
+                    jump = sts[1] - ens[0];
+                    len += ens[1] - sts[1];
+                }
+                slot |= 32u;
             }
         }
-        group_sync<WPC>();
-        // steps 2-4, chunk by chunk: a membership pass lists the members of ranks [lo, lo + CAP)
-        // (the first also counts them all), their runs are formed, and the kept members vote
-        unsigned best = 0u, votes = 0u;
-        int rlo = INT_MAX, rhi = -1;
-        int lo = 0;
-        auto to_chunk = [&](int r, int p, unsigned kd, float z) {
-            if (r >= lo && r < lo + CAP) S.par[r - lo] = make_int4(p, (int)kd, __float_as_int(z), 0);
+        const int incl = warp_incl_scan(len);
+        const int excl = incl - len;
+        const int T = __shfl_sync(0xFFFFFFFFu, incl, 31);
+        const unsigned ne = __ballot_sync(0xFFFFFFFFu, len > 0);
+        __syncwarp();   // the last group's readers are done
+        S.zco[lane] = zc;
+        if (len > 0) {
+            const int q = __popc(ne & lanes_below());
+            S.seg[q] = make_int4(st - excl, excl + n0, __float_as_int(g), jump);
+            S.seg_slot[q] = (unsigned char)slot;
+        }
+        const int my_start = len > 0 ? excl : INT_MAX;
+        __syncwarp();
+
+        // the hit at flattened index base + lane: its staged position, slot, g, f and whether that has
+        // to lie below g
+        auto locate = [&](int base, int &p, unsigned &sl, float &f, float &gq, bool &after) {
+            const int qb = __popc(__ballot_sync(0xFFFFFFFFu, my_start <= base)) - 1;   // the range owning base
+            const int d = my_start - base;
+            const unsigned bits = __reduce_or_sync(0xFFFFFFFFu, (d > 0 && d < 32) ? 1u << d : 0u);
+            const int q = qb + __popc(bits & upto);
+            const int4 sg = S.seg[q];
+            sl = S.seg_slot[q];
+            const int idx = base + lane;
+            after = idx >= sg.y;
+            gq = __int_as_float(sg.z);
+            p = sg.x + idx + (after ? sg.w : 0);
+            f = idx < T ? __ldg(&w.fsort[p]) : 0.f;
         };
-        const int n = scan_members<WPC, CAP, MAXP, NL, GEN, true>(ax, w, S, hot, fsort, zsort, cold, i, j, s32, refine_eps,
-                                                             to_chunk);
-        int written = n, listed = 0;   // members in the pool slot / written by step 3
-        int32_t *pool = nullptr;
-        if (KEEP && w.keep_members) {
-            // the event's member pool is shared by all its candidates: the count known, a slot is
-            // reserved now, and the runs' pass lists each member as it reads the member's entry
-            if (tid == 0) {
-                const unsigned reserved = n ? atomicAdd(&w.stats[ev].pool_used, (unsigned)n) : 0u;
-                const long long room = (long long)w.max_members - (long long)reserved;
-                S.pool_base = (int)min((long long)reserved, (long long)w.max_members);
-                S.pool_written = n ? (int)max(0LL, min((long long)n, room)) : 0;
+        auto is_member = [&](int base, int p, unsigned sl, float f, float gq, bool after) {
+            bool mem = (f < gq) == after;
+            if (GEN) {
+                const unsigned ij = __shfl_sync(0xFFFFFFFFu, rec.ij, (int)(sl & 31u));
+                if (base + lane < T && (sl & 32u))
+                    mem = general_member(ax, w, w.hot, w.cold, p, (int)(ij >> 16), (int)(ij & 0xFFFFu), s32, refine_eps);
             }
-            group_sync<WPC>();
-            const int base = S.pool_base;
-            written = S.pool_written;
-            if (tid == 0) {
-                w.mem_start[(int64_t)ev * w.max_cand + c] = base;
-                w.mem_count[(int64_t)ev * w.max_cand + c] = written;
+            return mem && base + lane < T;
+        };
+
+        // member lists of a context: a pool slot per candidate, reserved once its members are counted
+        // (lane k holds candidate k's count, base and entries written; in a team, lane 0 the warp's
+        // own part of them)
+        int cnt = 0, pool_base = 0, pool_n = 0;
+        auto count_window = [&](bool mem, unsigned sl) {
+            const int kq = (int)(sl & 31u) / NL;
+            for (int k = 0; k < C; ++k) {
+                const int c = __popc(__ballot_sync(0xFFFFFFFFu, mem && kq == k));
+                if (lane == k) cnt += c;
             }
-            pool = w.mem_pool + (int64_t)ev * w.max_members + base;
-            listed = written;
-        }
-        while (lo < n) {
-            if (lo > 0) {
-                group_sync<WPC>();   // the previous chunk's votes have read its members
-                scan_members<WPC, CAP, MAXP, NL, GEN, true>(ax, w, S, hot, fsort, zsort, cold, i, j, s32, refine_eps, to_chunk);
-            }
-            group_sync<WPC>();   // the chunk's list is complete
-            const ChunkOut co = chunk_runs<WPC, CAP, MAXP, NL, GEN, KEEP>(ax, S, cold, i, min(n - lo, CAP), rlo, rhi, pool,
-                                                                          lo, listed);
-            group_sync<WPC>();   // its runs and start bits are complete
-            vote_pairs<WPC, CAP, MAXP, NL, P10>(ax, S, grid, co.npairs, best, votes);
-            lo += co.consumed;
-        }
-        // step 5: the group's best key and votes, the final mask of its cell, the touched rows cleared
-        best = __reduce_max_sync(0xFFFFFFFFu, best);
-        votes = __reduce_add_sync(0xFFFFFFFFu, votes);
-        rlo = (int)__reduce_min_sync(0xFFFFFFFFu, (unsigned)rlo);
-        rhi = (int)__reduce_max_sync(0xFFFFFFFFu, (unsigned)(rhi + 1)) - 1;
-        if (WPC > 1) {   // the warps' results combined in one exchange
-            if (lane == 0) {
-                S.wtmp[4 * wg] = (int)best;
-                S.wtmp[4 * wg + 1] = (int)votes;
-                S.wtmp[4 * wg + 2] = rlo;
-                S.wtmp[4 * wg + 3] = rhi;
-            }
-            __syncthreads();
+        };
+        auto reserve = [&]() {
+            if (TEAM) {
+                if (lane == 0) team->members[wpos] = cnt;
+                __syncthreads();
+                int before = 0, all = 0;
 #pragma unroll
-            for (int k = 0; k < WPC; ++k) {
-                best = max(best, (unsigned)S.wtmp[4 * k]);
-                votes += k == wg ? 0u : (unsigned)S.wtmp[4 * k + 1];
-                rlo = min(rlo, S.wtmp[4 * k + 2]);
-                rhi = max(rhi, S.wtmp[4 * k + 3]);
-            }
-            __syncthreads();
-        }
-        group_sync<WPC>();   // every vote has landed
-        const unsigned cell = best ? 0xFFFFu - (best & 0xFFFFu) : 0u;
-        const uint32_t mask2 = best ? grid_mask<P10>(grid, cell) : 0u;
-        group_sync<WPC>();   // read before the clear
-        clear_rows<WPC, P10>(ax, grid, rlo, rhi);
-        if (tid == 0) {
-            hough_candidate out = cd;
-            out.n_members = (uint32_t)n;
-            out.icot = cell / (unsigned)ax.n_z0;
-            out.jz0 = cell % (unsigned)ax.n_z0;
-            out.mask2 = mask2;
-            out.flags = ((int)(best >> 16) >= min(ax.threshold, ax.n_layers) ? 1u : 0u) | (written < n ? 2u : 0u);
-            store_candidate(cands + c, out);
-            if (ev != acc_e) {
-                if (acc_e >= 0) {
-                    if (acc_members) atomicAdd(&w.stats[acc_e].n_members, acc_members);
-                    if (acc_votes) atomicAdd(&w.stats[acc_e].stage2_votes, acc_votes);
+                for (int k = 0; k < kWarps; ++k) {
+                    before += k < wpos ? team->members[k] : 0;
+                    all += team->members[k];
                 }
-                acc_e = ev;
-                acc_members = 0u;
-                acc_votes = 0ull;
+                if (threadIdx.x == 0) {
+                    const unsigned reserved = all ? atomicAdd(&w.stats[0].pool_used, (unsigned)all) : 0u;
+                    const long long room = (long long)w.max_members - (long long)reserved;
+                    team->pool_base = (int)min((long long)reserved, (long long)w.max_members);
+                    team->pool_n = all ? (int)max(0LL, min((long long)all, room)) : 0;
+                    w.mem_start[f0] = team->pool_base;
+                    w.mem_count[f0] = team->pool_n;
+                }
+                __syncthreads();
+                pool_base = team->pool_base + before;
+                pool_n = max(0, team->pool_n - before);
+            } else if (lane < C && f0 + lane < total) {
+                const unsigned reserved = cnt ? atomicAdd(&w.stats[0].pool_used, (unsigned)cnt) : 0u;
+                const long long room = (long long)w.max_members - (long long)reserved;
+                pool_base = (int)min((long long)reserved, (long long)w.max_members);
+                pool_n = cnt ? (int)max(0LL, min((long long)cnt, room)) : 0;
+                w.mem_start[f0 + lane] = pool_base;
+                w.mem_count[f0 + lane] = pool_n;
             }
-            acc_members += (unsigned)n;
-            acc_votes += (unsigned long long)votes;
+        };
+        // the candidate being voted: its best key and members so far
+        int cur = 0;
+        unsigned best = 0u;
+        int n_members = 0;
+        // the record of the lane's candidate, kept by the lanes of its first layer
+        unsigned r_best = 0u, r_mask2 = 0u;
+        int r_members = 0;
+        const bool one_event = __all_sync(0xFFFFFFFFu, rec.e == acc_e || rec.mask == 0u);
+        // step 5
+        auto finish = [&]() {
+            best = __reduce_max_sync(0xFFFFFFFFu, best);
+            acc_members += (unsigned)n_members;
+            if (TEAM) {
+                if (lane == 0) {
+                    team->best[wpos] = best;
+                    team->members[wpos] = n_members;
+                }
+                __syncthreads();   // every vote has landed
+                n_members = 0;
+#pragma unroll
+                for (int k = 0; k < kWarps; ++k) {
+                    best = max(best, team->best[k]);
+                    n_members += team->members[k];
+                }
+            } else {
+                __syncwarp();   // every vote has landed
+            }
+            uint32_t mask2 = 0u;
+            if (best) {
+                mask2 = grid_mask<P10>(grid, 0xFFFFu - (best & 0xFFFFu));
+                if (TEAM) __syncthreads(); else __syncwarp();   // read before the clear
+                uint4 *g4 = reinterpret_cast<uint4 *>(grid) + lane;
+                if (TEAM) {
+                    for (int q = threadIdx.x; q < grid_vecs; q += 32 * kWarps)
+                        reinterpret_cast<uint4 *>(grid)[q] = make_uint4(0u, 0u, 0u, 0u);
+                } else if (G64) {
+                    constexpr int kVecs = ((P10 ? (64 * 64 + 2) / 3 : 64 * 64 / 2) + 3) / 4;
+#pragma unroll
+                    for (int q = 0; q < kVecs; q += 32)
+                        if (q + 32 <= kVecs || lane < kVecs - q) g4[q] = make_uint4(0u, 0u, 0u, 0u);
+                } else {
+#pragma unroll 1
+                    for (int q = lane; q < grid_vecs; q += 32, g4 += 32) *g4 = make_uint4(0u, 0u, 0u, 0u);
+                }
+            }
+            if (lane == cur * NL) {
+                r_best = best;
+                r_mask2 = mask2;
+                r_members = n_members;
+            }
+            ++cur;
+            best = 0u;
+            n_members = 0;
+            if (TEAM) __syncthreads(); else __syncwarp();   // the grid is clear
+        };
+
+        // step 2: the members among the hits at base + lane, listed behind the nm there are; a lane's
+        // place in the list is given by ballots
+        int nm = 0;
+        auto append = [&](bool mem, int p, unsigned sl) {
+            const unsigned b = __ballot_sync(0xFFFFFFFFu, mem);
+            if (mem) {
+                const int r = nm + __popc(b & lanes_below());
+                S.list_p[r] = p;
+                S.list_slot[r] = (unsigned char)sl;
+            }
+            nm += __popc(b);
+        };
+        // the first windows' loads are all in flight before the first test
+        int h = 32 * wpos;   // the next window's first hit
+        {
+            int p[kListCap / 32];
+            unsigned sl[kListCap / 32];
+            float f[kListCap / 32], gq[kListCap / 32];
+            bool after[kListCap / 32];
+#pragma unroll
+            for (int u = 0; u < kListCap / 32; ++u)
+                if (h + 32 * TW * u < T) locate(h + 32 * TW * u, p[u], sl[u], f[u], gq[u], after[u]);
+#pragma unroll
+            for (int u = 0; u < kListCap / 32; ++u) {
+                if (h + 32 * TW * u < T) {
+                    const bool mem = is_member(h + 32 * TW * u, p[u], sl[u], f[u], gq[u], after[u]);
+                    append(mem, p[u], sl[u]);
+                    if (KEEP) count_window(mem, sl[u]);
+                }
+            }
+            h += 32 * TW * (kListCap / 32);
         }
-        group_sync<WPC>();   // the grid is clear and the scratch free for the next candidate
+        bool counting = KEEP;   // windows from here on are counted as they are first tested
+        for (;;) {
+            // more windows while the list has room for one
+            while (h < T && nm <= kListCap - 32) {
+                int p;
+                unsigned sl;
+                float f, gq;
+                bool after;
+                locate(h, p, sl, f, gq, after);
+                const bool mem = is_member(h, p, sl, f, gq, after);
+                append(mem, p, sl);
+                if (KEEP && counting) count_window(mem, sl);
+                h += 32 * TW;
+            }
+            if (KEEP && counting) {
+                // the members of the windows that wait for the list, then the candidates' pool slots
+                for (int base = h; base < T; base += 32 * TW) {
+                    int p;
+                    unsigned sl;
+                    float f, gq;
+                    bool after;
+                    locate(base, p, sl, f, gq, after);
+                    count_window(is_member(base, p, sl, f, gq, after), sl);
+                }
+                reserve();
+                counting = false;
+            }
+            __syncwarp();   // the list is complete
+            for (int r0 = 0; r0 < nm; r0 += 32) {
+                // step 3: coefficients and run of each of the round's members (a lane past the list
+                // repeats an entry and is dropped)
+                const int nr = min(32, nm - r0);
+                const bool valid = lane < nr;
+                const int at = r0 + min(lane, nr - 1);
+                const int p = S.list_p[at];
+                const unsigned sl = S.list_slot[at];
+                const float z = __ldg(&w.zsort[p]);
+                const int slot_r = (int)(sl & 31u);
+                const int k_r = slot_r / NL, l_r = slot_r - k_r * NL;
+                const float4 zcr = S.zco[slot_r];
+                float rb = zcr.z > 0.f ? __fdividef(1.f, zcr.z) : 0.f;   // approximate suffices
+                float a, b, mref, lo;
+                int len_r;
+                table_coefficients(ax, zcr, rb, z, &a, &b, &mref);
+                if (GEN) {
+                    const int i_r = (int)(__shfl_sync(0xFFFFFFFFu, rec.ij, slot_r) >> 16);
+                    if (sl & 32u) {
+                        exact_coefficients(ax, i_r, w.cold[p], &a, &b, &mref);
+                        rb = b > 0.f ? __frcp_rn(b) : 0.f;
+                    }
+                }
+                member_run(n_cotf, n_z0f, a, b, rb, mref, &lo, &len_r);
+                if (!valid) len_r = 0;
+                const int incl_r = warp_incl_scan(len_r);
+                const int st_r = incl_r - len_r;
+                const unsigned bkeep = __ballot_sync(0xFFFFFFFFu, len_r > 0);
+                const int last_word = (__shfl_sync(0xFFFFFFFFu, incl_r, 31) >> 5) + 1;
+                if (lane <= last_word) starts[lane] = 0u;
+#pragma unroll 1
+                for (int q = lane + 32; q <= last_word; q += 32) starts[q] = 0u;
+                __syncwarp();
+                if (len_r > 0) {
+                    const float c0 = lo - (float)st_r;
+                    S.par[__popc(bkeep & lanes_below())] = make_int4(
+                        __float_as_int(a), __float_as_int(b), __float_as_int(c0 - mref), (((int)c0 * n_z0) << 5) | l_r);
+                    atomicOr(&starts[st_r >> 5], 1u << (st_r & 31));
+                }
+                __syncwarp();
+                // step 4, a candidate's members at a time
+                for (int s0 = 0; s0 < nr;) {
+                    const int k = __shfl_sync(0xFFFFFFFFu, k_r, s0);
+                    const int s1 = s0 + __popc(__ballot_sync(0xFFFFFFFFu, valid && k_r == k));
+                    while (cur < k) finish();
+                    if (!one_event) {
+                        const int e = __shfl_sync(0xFFFFFFFFu, rec.e, k * NL);
+                        if (e != acc_e) flush(e);
+                    }
+                    if (KEEP) {
+                        const int base = __shfl_sync(0xFFFFFFFFu, pool_base, k), n = __shfl_sync(0xFFFFFFFFu, pool_n, k);
+                        const int r = n_members + lane - s0;   // the member's rank among its candidate's
+                        if (lane >= s0 && lane < s1 && r < n) w.mem_pool[base + r] = p;
+                    }
+                    n_members += s1 - s0;
+                    const int v0 = __shfl_sync(0xFFFFFFFFu, st_r, s0), v1 = __shfl_sync(0xFFFFFFFFu, incl_r, s1 - 1);
+                    // owner of a pair: the kept members before the candidate's, plus the runs starting at
+                    // or before the pair, less one
+                    const int4 *owner0 = S.par + (__popc(bkeep & ((1u << s0) - 1u)) - 1);
+                    const unsigned *sw = starts + (v0 >> 5);
+                    float row = (float)(v0 + lane);
+                    unsigned cv = (unsigned)((v0 + lane) * n_z0);
+                    unsigned word0 = *sw;
+#pragma unroll 1
+                    for (int left = v1 - v0 - lane; left > -lane; left -= 32) {   // (left + lane: the pairs to go)
+                        const unsigned word1 = *++sw;
+                        const unsigned bits = __funnelshift_r(word0, word1, v0);
+                        word0 = word1;
+                        const int4 pr = owner0[__popc(bits & upto)];
+                        owner0 += __popc(bits);
+                        // w(m) at the pair's row; its floor from the sum with 2^23 rounded down: below 0 that
+                        // falls under the bits of 2^23, above n_z0 it stays above n_z0
+                        const float wv = fmaf(-(row + __int_as_float(pr.z)), __int_as_float(pr.y), __int_as_float(pr.x));
+                        const unsigned n = (unsigned)__float_as_int(__fadd_rd(wv, 8388608.f)) - 0x4B000000u;
+                        const unsigned cell = cv + (unsigned)(pr.w >> 5) + n;
+                        const unsigned word = P10 ? __umulhi(cell, 0x55555556u) : cell >> 1;   // cell < 2^15: cell / 3
+                        const unsigned shift = P10 ? cell * 10u - word * 30u : (cell & 1u) << 4;
+                        const unsigned bit = __funnelshift_l(0u, 1u, pr.w);   // 1 << (pr.w & 31)
+                        // the vote and its judgement, predicated on the pair being in range
+                        asm volatile(
+                            "{\n\t.reg .pred p;\n\t.reg .b32 o, k;\n\t"
+                            "setp.lt.u32 p, %2, %3;\n\t"
+                            "setp.gt.and.s32 p, %4, 0, p;\n\t"
+                            "@p atom.shared.or.b32 o, [%5], %6;\n\t"
+                            "shr.u32 o, o, %7;\n\t"
+                            "lop3.b32 o, o, %8, %9, 0xEA;\n\t"   // (o & field) | bit
+                            "popc.b32 k, o;\n\t"
+                            "mad.lo.u32 k, k, 65536, %10;\n\t"
+                            "@p max.u32 %0, %0, k;\n\t"
+                            "@p add.u32 %1, %1, 1;\n\t}"
+                            : "+r"(best), "+r"(acc_votes)
+                            : "r"(n), "r"(n_z0), "r"(left), "r"(grid_s + word * 4u), "r"(bit << shift), "r"(shift),
+                              "r"(P10 ? 0x3FFu : 0xFFFFu), "r"(bit), "r"(0xFFFFu - cell)
+                            : "memory");
+                        row += 32.f;
+                        cv += 32u * (unsigned)n_z0;
+                    }
+                    s0 = s1;
+                }
+                __syncwarp();   // the round's entries are read before the next one's are written
+            }
+            if (h >= T) break;
+            nm = 0;
+        }
+        const int nc = min(C, total - f0);
+        while (cur < nc) finish();
+        const int written = !KEEP ? r_members : TEAM ? team->pool_n : __shfl_sync(0xFFFFFFFFu, pool_n, kc);
+        if (l == 0 && kc < nc && wpos == 0) {
+            const unsigned cell = r_best ? 0xFFFFu - (r_best & 0xFFFFu) : 0u;
+            // cell / n_z0: cell < 2^14 and n_z0 <= 256, so the quotient of the half-shifted cell stays
+            // far enough from a whole number for its roundings
+            const unsigned icot = G64 ? cell >> 6 : (unsigned)(((float)cell + 0.5f) * __frcp_rn(n_z0f));
+            hough_candidate out;
+            out.iq = (unsigned)i;
+            out.jphi = (unsigned)j;
+            out.mask = rec.mask;
+            out.n_members = (uint32_t)r_members;
+            out.icot = icot;
+            out.jz0 = cell - icot * (unsigned)n_z0;
+            out.mask2 = r_mask2;
+            out.flags = ((int)(r_best >> 16) >= min(ax.threshold, ax.n_layers) ? 1u : 0u) | (written < r_members ? 2u : 0u);
+            store_candidate(w.cands + f0 + kc, out);
+        }
     }
-    if (tid == 0 && acc_e >= 0) {
-        if (acc_members) atomicAdd(&w.stats[acc_e].n_members, acc_members);
-        if (acc_votes) atomicAdd(&w.stats[acc_e].stage2_votes, acc_votes);
-    }
+    flush(0);
 }
 
-// Membership and stage 2 of every candidate of every event, a group of WPC warps per candidate.
-template <int WPC, int CAP, int MAXP, int NL, bool P10>
-__global__ void __launch_bounds__(WPC == 1 ? 32 * kBatchGroups : 32 * WPC, WPC == 1 ? (P10 ? 8 : 5) : 1)
-    confirm_kernel(Axes ax, Workspace w, float s32, float refine_eps, int grid_words, int scratch_bytes,
-                   int bands_at, int many_groups, int many_scratch_bytes)
+// Membership and stage 2 of every candidate of every event.  EVENT: one event of a context, whose few
+// candidates are each shared by a CTA's warps.
+template <int NL, bool P10, bool G64, bool EVENT>
+__global__ void __launch_bounds__(32 * kWarps, P10 && !EVENT ? 7 : 5)
+    confirm_kernel(Axes ax, Workspace w, float s32, float refine_eps, int grid_words, int start_words, int group_warps,
+                   int chunk)
 {
     pdl_enter();
     extern __shared__ __align__(16) unsigned char smem_c[];
-    __shared__ LayerInfo s_info[HOUGH_MAX_LAYERS];
-    __shared__ int s_general;
-    const int ngroups = WPC == 1 ? (int)(blockDim.x >> 5) : 1;
-    const int gidx = WPC == 1 ? (int)(threadIdx.x >> 5) : 0;
-    Scratch<WPC, CAP, MAXP, NL> &S = *reinterpret_cast<Scratch<WPC, CAP, MAXP, NL> *>(smem_c + (size_t)gidx * scratch_bytes);
-    uint32_t *grid = reinterpret_cast<uint32_t *>(smem_c + (size_t)ngroups * scratch_bytes) + (size_t)gidx * grid_words;
-    // the layer records are requested first and stored last, so that their round trip overlaps the
-    // band counts' (or the candidate total's)
+    __shared__ int s_coarse[kBandChunks + 1];
+    __shared__ Team s_team;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // the layer records, one a lane
     LayerInfo li{};
-    if (threadIdx.x < HOUGH_MAX_LAYERS) li = w.info[threadIdx.x];
+    if (lane < ax.n_layers) li = w.info[lane];
+    const unsigned present = __ballot_sync(0xFFFFFFFFu, lane < ax.n_layers && li.present);
+    const unsigned general = __ballot_sync(0xFFFFFFFFu, lane < ax.n_layers && li.present && !li.uniform);
     // one event of a context whose candidate list was not compacted: every CTA scans the band counts
-    // into shared memory (behind the groups' scratch and grids) and reads its candidates from the
-    // band lists; the first CTA records the totals the compaction would have
+    // and reads its candidates from the band lists; the first CTA records the totals the compaction
+    // would have
     int total;
-    const int *band_offs = nullptr;
-    if (WPC > 1 && w.cands_from_bands) {   // (batches use one-warp groups and a compacted list)
-        int *bo = reinterpret_cast<int *>(smem_c + bands_at);
-        const int nb = n_bands(ax, w.band_rows);
-        const int found = block_excl_scan(w.band_counts, nb, bo);
+    const int *coarse = nullptr;
+    if (EVENT && w.cands_from_bands) {
+        const int found = scan_bands(w.band_counts, w.n_band_lists, chunk, s_coarse);
         total = min(found, w.max_cand);
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             w.stats[0].n_candidates = (unsigned)found;
@@ -886,61 +757,45 @@ __global__ void __launch_bounds__(WPC == 1 ? 32 * kBatchGroups : 32 * WPC, WPC =
             w.cand_base[1] = total;
             w.counters->total_cands = (unsigned)total;
         }
-        band_offs = bo;
+        coarse = s_coarse;
     } else {
         total = (int)w.counters->total_cands;
     }
-    if constexpr (WPC > 1) {
-        if (many_groups && total > kManyPerCta * (int)gridDim.x) {
-            // one event with many candidates (a fine grid, a busy event): each warp confirms its
-            // own candidates with its own scratch and grid, as in batches, instead of four warps
-            // sharing one candidate's chain
-            using S1 = Scratch<1, kBatchCap, kBatchPairs, NL>;
-            const int g = threadIdx.x >> 5, lane = threadIdx.x & 31;
-            S1 &s1 = *reinterpret_cast<S1 *>(smem_c + (size_t)g * many_scratch_bytes);
-            uint32_t *grid1 = reinterpret_cast<uint32_t *>(smem_c + (size_t)many_groups * many_scratch_bytes) +
-                              (size_t)g * grid_words;
-            if (g < many_groups) {
-                for (int q = lane; q < grid_words; q += 32) grid1[q] = 0u;
-                for (int q = lane; q < (int)(sizeof(S1) / 4); q += 32) reinterpret_cast<uint32_t *>(&s1)[q] = 0u;
-            }
-            if (threadIdx.x < HOUGH_MAX_LAYERS) s_info[threadIdx.x] = li;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                int gen = 0;
-                for (int l = 0; l < ax.n_layers; ++l) gen |= s_info[l].present && !s_info[l].uniform;
-                s_general = gen;
-            }
-            __syncthreads();
-            if (g >= many_groups) return;
-            if (s_general)
-                confirm_all<1, kBatchCap, kBatchPairs, NL, P10, true, true>(ax, w, s32, refine_eps, s1, grid1, s_info,
-                                                                            many_groups, g, total, band_offs);
-            else
-                confirm_all<1, kBatchCap, kBatchPairs, NL, P10, false, true>(ax, w, s32, refine_eps, s1, grid1, s_info,
-                                                                             many_groups, g, total, band_offs);
-            return;
-        }
+    const size_t scratch = sizeof(Scratch) + (size_t)start_words * 4;
+    if (EVENT && total <= kTeamRounds * (int)gridDim.x) {
+        if ((int)blockIdx.x >= total) return;
+        Scratch &S = *reinterpret_cast<Scratch *>(smem_c + warp * scratch);
+        unsigned *starts = reinterpret_cast<unsigned *>(&S + 1);
+        uint32_t *grid = reinterpret_cast<uint32_t *>(smem_c + kWarps * scratch);
+        for (int q = threadIdx.x; q < grid_words >> 2; q += 32 * kWarps)
+            reinterpret_cast<uint4 *>(grid)[q] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+        if (general)
+            confirm_groups<NL, P10, G64, true, true, true>(ax, w, s32, refine_eps, S, &s_team, starts, grid, grid_words >> 2, present,
+                                                     general, 1, blockIdx.x, gridDim.x, total, coarse, chunk);
+        else
+            confirm_groups<NL, P10, G64, false, true, true>(ax, w, s32, refine_eps, S, &s_team, starts, grid, grid_words >> 2, present,
+                                                      0u, 1, blockIdx.x, gridDim.x, total, coarse, chunk);
+        return;
     }
-    for (int q = group_tid<WPC>(); q < grid_words; q += 32 * WPC) grid[q] = 0u;
-    // the scratch starts zeroed: lanes past a list read its terms without a branch
-    for (int q = group_tid<WPC>(); q < (int)(sizeof(Scratch<WPC, CAP, MAXP, NL>) / 4); q += 32 * WPC)
-        reinterpret_cast<uint32_t *>(&S)[q] = 0u;
-    if (threadIdx.x < HOUGH_MAX_LAYERS) s_info[threadIdx.x] = li;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int g = 0;
-        for (int l = 0; l < ax.n_layers; ++l) g |= s_info[l].present && !s_info[l].uniform;
-        s_general = g;
-    }
-    __syncthreads();
-    // (one-warp kernels run batches, which keep no member lists)
-    if (s_general)
-        confirm_all<WPC, CAP, MAXP, NL, P10, true, (WPC > 1)>(ax, w, s32, refine_eps, S, grid, s_info, ngroups, gidx, total,
-                                                              band_offs);
+    // candidates per warp: as many as its lanes hold, fewer when that would leave warps without any;
+    // group q goes to CTA q mod gridDim, so that a few candidates spread over all SMs
+    if (warp >= group_warps) return;
+    const int nwarps = group_warps * gridDim.x;
+    const int C = max(1, min(32 / NL, total / nwarps));
+    const int first = warp * gridDim.x + blockIdx.x;
+    if ((int64_t)first * C >= total) return;
+    Scratch &S = *reinterpret_cast<Scratch *>(smem_c + warp * (scratch + (size_t)grid_words * 4));
+    unsigned *starts = reinterpret_cast<unsigned *>(&S + 1);
+    uint32_t *grid = starts + start_words;
+    for (int q = lane; q < grid_words >> 2; q += 32) reinterpret_cast<uint4 *>(grid)[q] = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+    if (general)
+        confirm_groups<NL, P10, G64, true, EVENT, false>(ax, w, s32, refine_eps, S, nullptr, starts, grid, grid_words >> 2, present,
+                                                  general, C, first, nwarps, total, coarse, chunk);
     else
-        confirm_all<WPC, CAP, MAXP, NL, P10, false, (WPC > 1)>(ax, w, s32, refine_eps, S, grid, s_info, ngroups, gidx, total,
-                                                               band_offs);
+        confirm_groups<NL, P10, G64, false, EVENT, false>(ax, w, s32, refine_eps, S, nullptr, starts, grid, grid_words >> 2, present,
+                                                   0u, C, first, nwarps, total, coarse, chunk);
 }
 
 __global__ void member_index_kernel(Workspace w, int32_t *idx_out, int64_t total)
@@ -973,7 +828,7 @@ int resident_ctas(K kernel, int threads, size_t smem, std::atomic<unsigned long 
     return n;
 }
 
-std::atomic<unsigned long long> g_ctas[4];
+std::atomic<unsigned long long> g_ctas[8];
 std::atomic<int> g_smem_optin{-1};
 
 int smem_optin()
@@ -988,34 +843,43 @@ int smem_optin()
     return m;
 }
 
-template <int WPC, int CAP, int MAXP, int NL, bool P10>
+template <int NL, bool P10, bool G64, bool EVENT>
 cudaError_t launch_confirm(const Axes &ax, const Workspace &w, int sms, float s32, float refine_eps,
                            cudaStream_t stream, std::atomic<unsigned long long> &memo)
 {
-    auto kernel = confirm_kernel<WPC, CAP, MAXP, NL, P10>;
+    auto kernel = confirm_kernel<NL, P10, G64, EVENT>;
     const int words = grid_words_for(ax, P10);
-    const size_t scratch = (sizeof(Scratch<WPC, CAP, MAXP, NL>) + 15) & ~(size_t)15;
-    const size_t per_group = scratch + (size_t)words * 4;
-    // one-warp groups: as many per CTA (up to kBatchGroups) as shared memory holds
-    const int room = smem_optin() - (int)(sizeof(LayerInfo) * HOUGH_MAX_LAYERS) - 1024;
-    const int groups = WPC == 1 ? std::max(1, std::min(kBatchGroups, room / (int)per_group)) : 1;
-    // a group of several warps may split into one-warp groups when its event has many candidates:
-    // room for WPC one-warp scratches and grids too, when they fit beside the bands
-    const size_t many_scratch = (sizeof(Scratch<1, kBatchCap, kBatchPairs, NL>) + 15) & ~(size_t)15;
-    const size_t many_bytes = (size_t)WPC * (many_scratch + (size_t)words * 4);
-    const int many = WPC > 1 && many_bytes <= 128 * 1024 ? WPC : 0;
-    const size_t layout = std::max((size_t)groups * per_group, many ? many_bytes : (size_t)0);
-    const size_t smem = layout + (w.cands_from_bands ? ((size_t)n_bands(ax, w.band_rows) + 1) * sizeof(int) : 0);
+    const int start_words = (ax.n_cot + 2 + 3) & ~3;   // 32 members' runs of at most n_cot rows
+    const size_t scratch = sizeof(Scratch) + (size_t)start_words * 4, grid = (size_t)words * 4;
+    // as many warps with a grid of their own per CTA (up to kWarps) as shared memory holds
+    const int room = smem_optin() - 2048;
+    const int warps = std::max(1, std::min(kWarps, room / (int)(scratch + grid)));
+    const size_t smem = std::max((size_t)warps * (scratch + grid), EVENT ? kWarps * scratch + grid : (size_t)0);
     cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (!err) err = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                          cudaSharedmemCarveoutMaxShared);
     if (err) return err;
-    const int threads = 32 * WPC * groups;
+    const int threads = 32 * (EVENT ? kWarps : warps);
     const int ctas = resident_ctas(kernel, threads, smem, memo);
+    const int chunk = (n_bands(ax, w.band_rows) + kBandChunks - 1) / kBandChunks;
     // the number of candidates is known on the device only: a persistent grid of exactly the
-    // resident CTAs, each group striding over the flattened (event, candidate) work
+    // resident CTAs, each warp striding over the flattened list
     return launch_chained(kernel, dim3(ctas * sms), dim3(threads), smem, stream, ax, w, s32, refine_eps, words,
-                          (int)scratch, (int)layout, many, (int)many_scratch);
+                          start_words, warps, chunk);
+}
+
+template <bool EVENT>
+cudaError_t launch_confirm_for(const Axes &ax, const Workspace &w, int sms, float refine_eps, cudaStream_t stream)
+{
+    const float s32 = (float)(ax.n_phi * kInvTwoPi);
+    std::atomic<unsigned long long> *memo = g_ctas + (EVENT ? 4 : 0);
+    // at most 10 layers: 10 lanes a candidate, the grid's masks packed three to a word
+    const bool g64 = ax.n_cot == 64 && ax.n_z0 == 64;
+    if (ax.n_layers <= 10)
+        return g64 ? launch_confirm<10, true, true, EVENT>(ax, w, sms, s32, refine_eps, stream, memo[0])
+                   : launch_confirm<10, true, false, EVENT>(ax, w, sms, s32, refine_eps, stream, memo[1]);
+    return g64 ? launch_confirm<16, false, true, EVENT>(ax, w, sms, s32, refine_eps, stream, memo[2])
+               : launch_confirm<16, false, false, EVENT>(ax, w, sms, s32, refine_eps, stream, memo[3]);
 }
 
 }  // namespace
@@ -1027,18 +891,9 @@ bool stage2_reads_bands(const Axes &ax, int band_rows) { return n_bands(ax, band
 cudaError_t launch_stage2(const Axes &ax, const Workspace &w, int sms, float refine_eps, cudaStream_t stream,
                           cudaEvent_t between)
 {
-    const float s32 = (float)(ax.n_phi * kInvTwoPi);
     if (w.keep_members && w.n_events != 1) return cudaErrorInvalidValue;   // only single events keep member lists
-    cudaError_t err;
-    if (w.n_events == 1) {
-        // one event: a few hundred candidates, each a chain of dependent steps, so four warps share one
-        err = launch_confirm<kEventWarps, kEventCap, kEventPairs, HOUGH_MAX_LAYERS, false>(ax, w, sms, s32, refine_eps, stream, g_ctas[0]);
-    } else if (ax.n_layers <= 10) {
-        // a batch: a warp per candidate, the grid's masks packed three to a word so more warps fit an SM
-        err = launch_confirm<1, kBatchCap, kBatchPairs, 10, true>(ax, w, sms, s32, refine_eps, stream, g_ctas[1]);
-    } else {
-        err = launch_confirm<1, kBatchCap, kBatchPairs, HOUGH_MAX_LAYERS, false>(ax, w, sms, s32, refine_eps, stream, g_ctas[2]);
-    }
+    cudaError_t err = w.keep_members ? launch_confirm_for<true>(ax, w, sms, refine_eps, stream)
+                                     : launch_confirm_for<false>(ax, w, sms, refine_eps, stream);
     if (err) return err;
     if (between && (err = cudaEventRecord(between, stream))) return err;
     return cudaSuccess;

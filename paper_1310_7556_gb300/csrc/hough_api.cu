@@ -81,6 +81,7 @@ struct hough_ctx {
     // the peak search left the candidate list uncompacted (stage 2 reads the band lists itself);
     // a call that reads the list or the counters before stage 2 compacts it first
     bool list_pending = false;
+    bool listed = false;                 // the event's candidate list was compacted (else stage 2 reads the band lists)
     bool timing = false;
     // 0 before staging, 1 after staging, 2 after the gather, 3 after the vote, 4 after the band
     // peaks, 5 after the candidate scan, 6 after stage 2
@@ -389,9 +390,10 @@ int enqueue_vote(hough_ctx *c, const float *r, const float *phi, const float *z,
 int settle_list(hough_ctx *c, cudaStream_t s)
 {
     if (!c->list_pending) return HOUGH_OK;
-    CU(launch_compact(c->ax, c->w, s), "candidate scan kernel");
-    g_launches += peak_launches(1) - 1;
+    CU(launch_compact(c->ax, c->w, s, true), "candidate scan kernel");
+    g_launches += kCompactLaunches;
     c->list_pending = false;
+    c->listed = true;
     return HOUGH_OK;
 }
 
@@ -498,7 +500,7 @@ int hough_create(const hough_geometry *geometry, const hough_binning *binning, c
     A(c->alloc(&w.zco, (size_t)ax.n_layers * ax.n_qpt));
     A(c->alloc(&w.kq32, ax.n_qpt));
     A(c->alloc(&w.M, (size_t)ax.n_qpt * ax.n_phi));
-    A(c->alloc(&w.cands, w.max_cand));
+    A(c->alloc(&w.cands, w.max_cand)); A(c->alloc(&w.cand_list, w.max_cand));
     A(c->alloc(&w.band_cands, band_list_entries_impl(ax)));
     A(c->alloc(&w.band_counts, n_bands(ax, 1))); A(c->alloc(&w.band_offs, n_bands(ax, 1)));
     A(c->alloc(&w.mem_start, w.max_cand)); A(c->alloc(&w.mem_count, w.max_cand));
@@ -518,7 +520,6 @@ int hough_create(const hough_geometry *geometry, const hough_binning *binning, c
     w.fused = 0;
     w.keep_members = 1;   // hough_get_members reads the member lists
     w.recycle = 1;
-    w.compact_in_peaks = 1;
     w.stats = c->stats_buf[0];
     w.radii = c->radii_buf[0];
     // FP32 q/pT bin centres: the FP64 centre rounded once
@@ -561,20 +562,18 @@ int hough_peaks(hough_ctx *c, void *stream)
     if (!c) return fail(HOUGH_EINVAL, "ctx is required");
     if (c->stage < 1) return fail(HOUGH_ENOTREADY, "hough_vote has not run");
     CU(cudaSetDevice(c->device), "cudaSetDevice");
-    // The candidate list: stage 2 reads the band lists itself when their offsets fit its shared
-    // memory (the list is compacted later only for a caller that reads it first); else the peak
-    // kernel's last CTA compacts it, except after the fused vote (whose peak kernel may not run).
+    // The candidate list: stage 2 reads the band lists itself when there are few enough of them (the
+    // list is compacted later only for a caller that reads it first); else it is compacted here.
     // Either way the peak kernel zeroes the bucket profile for the next event.
-    const bool fused = c->tiling.vote_mode == HOUGH_VOTE_FUSED;
-    const bool deferred = !fused && stage2_reads_bands(c->ax, c->tiling.band_rows);
-    c->w.compact_in_peaks = fused || deferred ? 0 : 1;
+    const bool deferred = stage2_reads_bands(c->ax, c->w.band_rows);
     CU(launch_band_peaks(c->ax, c->w, c->tiling, (cudaStream_t)stream), "peak kernel");
-    c->compacted = fused;   // a separate compaction kernel (the peak kernel's own last CTA is timed with it)
+    c->compacted = !deferred;
     if (c->timing) { CU(cudaEventRecord(c->ev[4], (cudaStream_t)stream), "event"); c->timed |= 16; }
-    if (fused) CU(launch_compact(c->ax, c->w, (cudaStream_t)stream), "candidate scan kernel");
+    if (!deferred) CU(launch_compact(c->ax, c->w, (cudaStream_t)stream, true), "candidate scan kernel");
     if (c->timing) { CU(cudaEventRecord(c->ev[5], (cudaStream_t)stream), "event"); c->timed |= 32; }
-    g_launches += fused ? peak_launches(1) : 1;
+    g_launches += deferred ? 1 : kPeakLaunches;
     c->list_pending = deferred;
+    c->listed = !deferred;
     c->clean = true;
     c->stage = 2;
     return HOUGH_OK;
@@ -585,7 +584,8 @@ int hough_stage2(hough_ctx *c, void *stream)
     if (!c) return fail(HOUGH_EINVAL, "ctx is required");
     if (c->stage < 2) return fail(HOUGH_ENOTREADY, "hough_peaks has not run");
     CU(cudaSetDevice(c->device), "cudaSetDevice");
-    c->w.cands_from_bands = c->list_pending ? 1 : 0;   // the confirmation compacts as it goes
+    c->w.cands_from_bands = c->listed ? 0 : 1;   // the confirmation compacts as it goes
+    c->w.n_band_lists = n_bands(c->ax, c->w.band_rows);
     CU(launch_stage2(c->ax, c->w, c->sms, c->refine_eps, (cudaStream_t)stream, c->timing ? c->ev[7] : nullptr),
        "stage-2 kernels");
     c->w.cands_from_bands = 0;
@@ -720,9 +720,9 @@ int hough_process(hough_ctx *c, const float *r, const float *phi, const float *z
     if ((rc = hough_peaks(c, stream))) return rc;
     if ((rc = hough_stage2(c, stream))) return rc;
     // one kernel writes both the candidates and the counters into mapped memory
-    CU(launch_pack_candidates(c->ax, c->w, c->cands_mapped_dev, s, std::min<long long>(cap, c->w.max_cand), nullptr,
-                              c->stats_mapped_dev, 152),
-       "pack kernel");
+    CU(launch_copy_candidates(c->w, c->cands_mapped_dev, s, std::min<long long>(cap, c->w.max_cand), c->stats_mapped_dev,
+                              152),
+       "copy kernel");
     g_launches += 1;
     CU(cudaStreamSynchronize(s), "synchronise");
     *c->stats_host = *c->stats_mapped;   // hough_get_stats and friends read the last event's copy

@@ -14,8 +14,10 @@
 //   tab[L*Nq] (8 B)           per (layer, q/pT row): Nphi asin(x) / (2 pi) = I + g, for layers whose
 //                             hits share one radius; arc[L*Nq] the arc length s (FP64)
 //   M[Nq*Nphi] (uint16)       stage-1 accumulator, row-major layer masks
-//   band_cands[n_bands*band_cap] (8 B)  peak candidates of each row band: cell index, mask
-//   cands[max_cand] (32 B)    hough_candidate records in raster order
+//   band_cands[n_bands*band_cap] (8 B)  peak candidates of each row band: row << 16 | column, mask
+//   cand_list (16 B)          the candidates of all events in order: row << 16 | column, mask, event,
+//                             the event's first hit; cands (32 B) their hough_candidate records, both
+//                             at the flattened index cand_base[e] + rank within the event
 //   mem_pool[max_members]     member hits (staged positions); mem_start/mem_count per candidate
 //                             (contexts only: a batch keeps no member lists)
 #pragma once
@@ -118,9 +120,8 @@ struct HitInputs {
 // Counters of a whole batch.
 struct BatchCounters {
     unsigned int total_cands;      // candidates kept over all events
-    unsigned int pad1;
-    unsigned int peaks_done;       // CTAs of the peak search finished (compaction in the last one)
-    unsigned int pad;
+    unsigned int scans_done;       // events whose band counts are scanned (the last one's CTA adds up the totals)
+    unsigned int pad[2];
 };
 
 // Device buffers of a batch of events that share one set of axes.
@@ -152,6 +153,7 @@ struct Workspace {
     uint2 *band_cands;            // n_events * n_bands * band_cap
     int32_t *band_counts;         // n_events * n_bands
     int32_t *band_offs;           // n_events * n_bands
+    uint4 *cand_list;             // n_events * max_cand
     hough_candidate *cands;       // n_events * max_cand
     int32_t *mem_pool;            // max_members: event-local staged positions (contexts only)
     int32_t *mem_start;           // max_cand (contexts only)
@@ -164,8 +166,8 @@ struct Workspace {
     int fused;                    // vote_mode HOUGH_VOTE_FUSED: the vote kernel searched the bands
     int keep_members;             // 1: confirmation writes member lists to mem_pool (contexts); 0: none (batches)
     int copy_wait;                // < 0: the first bound on a bulk-copy wait expires at once (a test of the error path)
-    int compact_in_peaks;         // one event: the peak kernel's last CTA compacts the candidate list
     int cands_from_bands;         // one event: the confirmation reads its candidates from the band lists
+    int n_band_lists;             // their number (set with it)
     // A context's state is left clean for its next event by the kernels that last use it, so that no
     // clearing kernel opens the next event: the hit sort zeroes the bucket counts, the peak search
     // the bucket profile, and the counting kernel the counters and radius ranges of the next event,
@@ -219,18 +221,17 @@ cudaError_t launch_stage(const Axes &ax, const Workspace &w, cudaStream_t stream
                          bool clear = true);
 cudaError_t launch_vote(const Axes &ax, const Workspace &w, const Tiling &t, float refine_eps,
                         cudaStream_t stream);
-cudaError_t launch_peaks(const Axes &ax, const Workspace &w, const Tiling &t, cudaStream_t stream);
-// The pieces of launch_vote and launch_peaks, for callers that time them separately.
+// The pieces of launch_vote, for callers that time them separately, and of the peak search.
 cudaError_t launch_gather(const Axes &ax, const Workspace &w, const Tiling &t, cudaStream_t stream);
 cudaError_t launch_scatter(const Axes &ax, const Workspace &w, const Tiling &t, float refine_eps, bool general_only,
                            cudaStream_t stream);
 cudaError_t launch_band_peaks(const Axes &ax, const Workspace &w, const Tiling &t, cudaStream_t stream);
-cudaError_t launch_compact(const Axes &ax, const Workspace &w, cudaStream_t stream);
-// All events' candidates concatenated: the first `limit` into `out` (device-accessible), the rest
-// into `rest` at the same indices when it is given, else dropped; the first event's counters to
+// The band lists into cand_list, the candidate counts and cand_base.  records: also write the
+// candidates' records with the stage-2 fields empty (a caller reads them before stage 2).
+cudaError_t launch_compact(const Axes &ax, const Workspace &w, cudaStream_t stream, bool records = false);
+// The first `limit` candidate records into `out` (device-accessible); the first event's counters to
 // `stats_out` (device-accessible) when it is given.
-cudaError_t launch_pack_candidates(const Axes &ax, const Workspace &w, hough_candidate *out, cudaStream_t stream,
-                                   long long limit = 1LL << 62, hough_candidate *rest = nullptr,
+cudaError_t launch_copy_candidates(const Workspace &w, hough_candidate *out, cudaStream_t stream, long long limit,
                                    DevStats *stats_out = nullptr, int blocks = 1216);
 cudaError_t launch_stage2(const Axes &ax, const Workspace &w, int sms, float refine_eps, cudaStream_t stream,
                           cudaEvent_t between = nullptr);
@@ -289,8 +290,9 @@ void note_launches(uint64_t n);
 // Kernels launched by each enqueue function (for hough_kernel_launches).
 constexpr int kStageLaunches = 4;
 constexpr int kVoteLaunches = 2;
-// peak search, compaction, and for batches of several events the candidate-base scan
-inline int peak_launches(int n_events) { return n_events == 1 ? 2 : 3; }
+// peak search, and the compaction's scan of the band counts and copy of the band lists
+constexpr int kCompactLaunches = 2;
+constexpr int kPeakLaunches = 1 + kCompactLaunches;
 constexpr int kStage2Launches = 1;
 
 // Exact FP64 helpers used by the staging, table and refinement code.  They evaluate the
@@ -529,8 +531,8 @@ __device__ __forceinline__ int wrap_col(int j, int n)
 // A cell with value p is a candidate when p >= threshold, the neighbours at (-1,-1), (-1,0),
 // (-1,+1), (0,-1) are below p and the other four are not above it; phi0 wraps.  Each thread tests
 // 8 consecutive cells per pass, so thread order is raster order and one block-wide scan of the
-// per-thread counts places every candidate.  Candidates go to `out` (cell index i * Nphi + j,
-// mask read from M) in raster order; returns their number.  Called by all TPB threads.
+// per-thread counts places every candidate.  Candidates go to `out` (row << 16 | column, mask read
+// from M) in raster order; returns their number.  Called by all TPB threads.
 // D3 (a grid with a d0 axis): the band's 3 x 3 x 3 blocks are held as three slices of nrows + 2
 // rows each -- slice m - 1, the band's own, slice m + 1 -- the band's rows in the middle one; the
 // nine neighbours of slice m - 1 precede a cell in raster order (strictly lower), the nine of
@@ -606,11 +608,11 @@ __device__ __forceinline__ int band_peak_search(const V *pc, int nrows, int i0, 
         while (pk) {
             const int c = __ffs(pk) - 1;
             pk &= pk - 1u;
-            const unsigned cellg = (unsigned)(i0 + rr) * (unsigned)nphi + (unsigned)(j0 + c);
             if (idx < cap)
-                out[idx] = make_uint2(cellg, MASKS   ? (unsigned)pc[(rr + 1) * nphi + j0 + c]
-                                             : SMASK ? (unsigned)M[rr * nphi + j0 + c]
-                                                     : (unsigned)M[cellg]);
+                out[idx] = make_uint2((unsigned)(i0 + rr) << 16 | (unsigned)(j0 + c),
+                                      MASKS   ? (unsigned)pc[(rr + 1) * nphi + j0 + c]
+                                      : SMASK ? (unsigned)M[rr * nphi + j0 + c]
+                                              : (unsigned)M[(int64_t)(i0 + rr) * nphi + j0 + c]);
             ++idx;
         }
         running += s_total;

@@ -32,7 +32,8 @@
 //    of the tile's window of buckets (gather_count_kernel).
 //
 // Peaks: candidates of each band of band_rows rows (one row by default) go to a band list in
-// raster order; a per-event scan then concatenates the band lists into the raster-ordered list.
+// raster order; a scan of the band counts and a copy then concatenate the band lists of all events
+// into one list.
 // With a d0 axis a band lies in one slice and its cells take the 3 x 3 x 3 rule (peaks3_kernel).
 #include <algorithm>
 #include <atomic>
@@ -1058,8 +1059,6 @@ __global__ void __launch_bounds__(TPB) gather_count_kernel(GatherParams p, int f
     }
 }
 
-__device__ void compact_if_last(const Axes &ax, const Workspace &w, void *buf, size_t buf_bytes);
-
 // A context's bucket profile is read for the last time by the vote, which the peak search follows:
 // zero it here for the next event (Workspace::recycle).
 __device__ __forceinline__ void recycle_profile(const Axes &ax, const Workspace &w)
@@ -1102,8 +1101,6 @@ __global__ void __launch_bounds__(kPeakThreads) peaks_kernel(Axes ax, Workspace 
         __syncthreads();
         const int cnt = band_peak_search<kPeakThreads>(pv, nrows, i0, nphi, ax.threshold, M, out, w.band_cap);
         if (threadIdx.x == 0) w.band_counts[(int64_t)e * nb + band] = cnt;
-        __syncthreads();   // the band buffer is free
-        compact_if_last(ax, w, pc, band_smem_bytes(ax, R));
         return;
     }
     uint16_t *pm = reinterpret_cast<uint16_t *>(pc + (size_t)(R + 2) * nphi);   // the band's own rows' masks
@@ -1126,8 +1123,6 @@ __global__ void __launch_bounds__(kPeakThreads) peaks_kernel(Axes ax, Workspace 
     const int cnt = band_peak_search<kPeakThreads, unsigned char, false, false, true>(pc, nrows, i0, nphi, ax.threshold,
                                                                                      pm, out, w.band_cap);
     if (threadIdx.x == 0) w.band_counts[(int64_t)e * nb + band] = cnt;
-    __syncthreads();   // the band buffer is free
-    compact_if_last(ax, w, pc, band_smem_bytes(ax, R));
 }
 
 // Peak search of one band of band_rows q/pT rows of one d0 slice m of a grid with a d0 axis: the
@@ -1182,199 +1177,121 @@ __global__ void __launch_bounds__(kPeakThreads) peaks3_kernel(Axes ax, Workspace
         cnt = band_peak_search<kPeakThreads, unsigned char, true>(pc, nrows, row0, nphi, ax.threshold, M, out,
                                                                   w.band_cap);
     if (threadIdx.x == 0) w.band_counts[(int64_t)e * nb + band] = cnt;
-    __syncthreads();   // the band buffer is free
-    compact_if_last(ax, w, pc, band_smem_bytes(ax, R));
 }
 
-// One event's candidate list: exclusive scan of the band counts, then the band lists concatenated
-// into the raster-ordered candidate list (the first max_cand of them).  With the band offsets in
-// shared memory every thread copies candidates by their index (the band found by binary search
-// over the offsets), so the copy costs one round trip however the candidates fall into bands.
-// `parts` CTAs may share an event, each copying its slice (this one is `part`); part 0 also records
-// the event's totals (and handles band counts too many to stage).  `single`: the batch is one
-// event, whose flattened candidate base this CTA then writes itself.  Called by all TPB threads.
-// The band offsets are staged in shared memory when they fit (`offs_smem`, `offs_cap` entries);
-// otherwise they go through device memory and a warp copies a band at a time.
-constexpr int kCompactSmemBands = 4096;
-
-template <int TPB>
-__device__ void compact_event(const Axes &ax, const Workspace &w, int e, int part, int parts, int single,
-                              int *s_offs, int offs_cap)
+// Exclusive scan over the CTA (kCompactThreads threads); *total receives the sum.  Every thread takes part.
+__device__ __forceinline__ int block_excl(int v, int *total)
 {
-    __shared__ int s_warp[TPB / 32];
-    const int nb = n_bands(ax, w.band_rows);
-    const bool staged = nb + 1 <= offs_cap;
-    const int32_t *counts = w.band_counts + (int64_t)e * nb;
-    int32_t *offs = w.band_offs + (int64_t)e * nb;
+    __shared__ int s_warp[kCompactThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int chunk = (nb + TPB - 1) / TPB;
-    const int k0 = min(nb, (int)threadIdx.x * chunk), k1 = min(nb, k0 + chunk);
-    int sum = 0;
-    for (int k = k0; k < k1; ++k) sum += counts[k];
-    int incl = sum;
+    int incl = v;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
         const int t = __shfl_up_sync(0xFFFFFFFFu, incl, d);
         if (lane >= d) incl += t;
     }
+    __syncthreads();   // the last call's readers are done
     if (lane == 31) s_warp[warp] = incl;
     __syncthreads();
-    if (warp == 0) {
-        int wv = lane < TPB / 32 ? s_warp[lane] : 0;
+    int wi = s_warp[lane];
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int t = __shfl_up_sync(0xFFFFFFFFu, wv, d);
-            if (lane >= d) wv += t;
-        }
-        if (lane < TPB / 32) s_warp[lane] = wv;
+    for (int d = 1; d < 32; d <<= 1) {
+        const int t = __shfl_up_sync(0xFFFFFFFFu, wi, d);
+        if (lane >= d) wi += t;
     }
-    __syncthreads();
-    int run = (warp > 0 ? s_warp[warp - 1] : 0) + incl - sum;
-    for (int k = k0; k < k1; ++k) {
-        if (staged) s_offs[k] = run;
-        else if (part == 0) offs[k] = run;
-        run += counts[k];
-    }
-    const int total = s_warp[TPB / 32 - 1];
-    const int kept = min(total, w.max_cand);
-    if (part == 0 && threadIdx.x == 0) {
-        w.stats[e].n_candidates = (unsigned)total;
-        if (total > w.max_cand) atomicOr(&w.stats[e].device_error, HOUGH_DEVERR_CAND);
-        if (single) {
-            w.cand_base[0] = 0;
-            w.cand_base[1] = kept;
-            w.counters->total_cands = (unsigned)kept;
-        }
-    }
-    __syncthreads();
-    hough_candidate *cands = w.cands + (int64_t)e * w.max_cand;
-    const uint2 *lists = w.band_cands + (int64_t)e * nb * w.band_cap;
-    auto emit = [&](int c, uint2 v) {
-        hough_candidate cd;
-        cd.iq = v.x / (unsigned)ax.n_phi;
-        cd.jphi = v.x % (unsigned)ax.n_phi;
-        cd.mask = v.y;
-        cd.n_members = 0u;
-        cd.icot = cd.jz0 = cd.mask2 = cd.flags = 0u;
-        cands[c] = cd;
-    };
-    if (staged) {
-        const int per = (kept + parts - 1) / parts;
-        const int c_end = min(kept, (part + 1) * per);
-        for (int c = part * per + threadIdx.x; c < c_end; c += TPB) {
-            // the band holding candidate c: the last b with offs[b] <= c (empty bands share offsets)
-            int lo = 0, hi = nb - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (s_offs[mid] <= c) lo = mid; else hi = mid - 1;
-            }
-            emit(c, lists[(int64_t)lo * w.band_cap + (c - s_offs[lo])]);
-        }
-        return;
-    }
-    if (part != 0) return;
-    __syncthreads();   // the offsets in device memory are complete
-    for (int b = warp; b < nb; b += TPB / 32) {
-        const int n = counts[b], o = offs[b];
-        for (int k = lane; k < n; k += 32) {
-            const int c = o + k;
-            if (c >= w.max_cand) break;
-            emit(c, lists[(int64_t)b * w.band_cap + k]);
-        }
-    }
+    *total = __shfl_sync(0xFFFFFFFFu, wi, 31);
+    return incl - v + (warp > 0 ? __shfl_sync(0xFFFFFFFFu, wi, warp - 1) : 0);
 }
 
-__global__ void __launch_bounds__(kCompactThreads) compact_kernel(Axes ax, Workspace w, int single, int parts)
+// Compaction, first launch, one CTA per event: the exclusive scan of its band counts (band_offs) and
+// its number of candidates; the CTA that finishes last adds up the kept candidates of the events
+// before each one (cand_base), so that later kernels can spread all events' candidates over the
+// whole device.
+__global__ void __launch_bounds__(kCompactThreads) band_scan_kernel(Axes ax, Workspace w)
 {
     pdl_enter();
-    __shared__ int s_offs[kCompactSmemBands + 1];
-    compact_event<kCompactThreads>(ax, w, blockIdx.x / parts, blockIdx.x % parts, parts, single, s_offs,
-                                   kCompactSmemBands + 1);
-}
-
-// One event in one context: the CTA of the peak search that finishes last compacts the candidate
-// list itself, saving the launch of the compaction (the band counts and lists of every CTA are
-// visible to it after their fences).  Its band buffer (`buf`, `buf_bytes`), no longer needed,
-// holds the band offsets.
-__device__ void compact_if_last(const Axes &ax, const Workspace &w, void *buf, size_t buf_bytes)
-{
     __shared__ int s_last;
-    if (!w.compact_in_peaks) return;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(&w.counters->peaks_done, 1u) == gridDim.x - 1;
+    const int e = blockIdx.x, nb = n_bands(ax, w.band_rows);
+    const int32_t *counts = w.band_counts + (int64_t)e * nb;
+    int32_t *offs = w.band_offs + (int64_t)e * nb;
+    int carry = 0;
+    for (int b0 = 0; b0 < nb; b0 += kCompactThreads) {
+        const int b = b0 + threadIdx.x;
+        int sum;
+        const int excl = block_excl(b < nb ? counts[b] : 0, &sum);
+        if (b < nb) offs[b] = carry + excl;
+        carry += sum;
+    }
+    if (threadIdx.x == 0) {
+        w.stats[e].n_candidates = (unsigned)carry;
+        if (carry > w.max_cand) atomicOr(&w.stats[e].device_error, HOUGH_DEVERR_CAND);
+        __threadfence();
+        s_last = atomicAdd(&w.counters->scans_done, 1u) == gridDim.x - 1;
+    }
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    compact_event<kPeakThreads>(ax, w, 0, 0, 1, 1, static_cast<int *>(buf), (int)(buf_bytes / sizeof(int)));
-    if (threadIdx.x == 0) w.counters->peaks_done = 0u;   // ready for the next event
-}
-
-// One CTA: the first flattened candidate index of every event (kept candidates only), so that
-// later kernels can spread all events' candidates over the whole device.
-__global__ void __launch_bounds__(kCompactThreads) cand_scan_kernel(Workspace w)
-{
-    pdl_enter();
-    __shared__ int s_warp[kCompactThreads / 32];
-    __shared__ int s_carry;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x == 0) s_carry = 0;
-    __syncthreads();
-    for (int base = 0; base < w.n_events; base += kCompactThreads) {
-        const int e = base + threadIdx.x;
-        const int v = e < w.n_events ? (int)min((unsigned)w.max_cand, w.stats[e].n_candidates) : 0;
-        int incl = v;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int t = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-            if (lane >= d) incl += t;
-        }
-        if (lane == 31) s_warp[warp] = incl;
-        __syncthreads();
-        if (warp == 0) {
-            const int sv = s_warp[lane];
-            int si = sv;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const int t = __shfl_up_sync(0xFFFFFFFFu, si, d);
-                if (lane >= d) si += t;
-            }
-            s_warp[lane] = si - sv;
-        }
-        __syncthreads();
-        const int excl = s_carry + s_warp[warp] + incl - v;
-        if (e < w.n_events) w.cand_base[e] = excl;
-        __syncthreads();
-        if (threadIdx.x == kCompactThreads - 1) s_carry = excl + v;
-        __syncthreads();
+    int base = 0;
+    for (int e0 = 0; e0 < w.n_events; e0 += kCompactThreads) {
+        const int ev = e0 + threadIdx.x;
+        int sum;
+        const int kept = ev < w.n_events ? (int)min((unsigned)w.max_cand, __ldcg(&w.stats[ev].n_candidates)) : 0;
+        const int excl = block_excl(kept, &sum);
+        if (ev < w.n_events) w.cand_base[ev] = base + excl;
+        base += sum;
     }
     if (threadIdx.x == 0) {
-        w.cand_base[w.n_events] = s_carry;
-        w.counters->total_cands = (unsigned)s_carry;
+        w.cand_base[w.n_events] = base;
+        w.counters->total_cands = (unsigned)base;
+        w.counters->scans_done = 0u;   // ready for the next event
     }
 }
 
-// All events' candidate lists, concatenated in event order into `out` (positions from cand_base).
-// (the first `limit` to `out`, the rest -- when `rest` is given -- to rest at the same index)
-// When `stats_out` is given, block 0 also copies the first event's counters there.
-__global__ void pack_candidates_kernel(Workspace w, hough_candidate *out, long long limit, hough_candidate *rest,
-                                       DevStats *stats_out)
+// Compaction, second launch: a warp per band copies its list to the flattened one (and, with
+// `records`, to candidate records whose stage-2 fields are empty).  Bound by the 16-byte entries it
+// writes; a CTA per part of an event that searched the bands of each candidate and wrote 32-byte
+// records took 310 us for the 7.5M candidates of a 256-event batch.
+__global__ void __launch_bounds__(256) band_copy_kernel(Axes ax, Workspace w, int records)
+{
+    pdl_enter();
+    const int nb = n_bands(ax, w.band_rows);
+    const int lane = threadIdx.x & 31;
+    const int64_t bands = (int64_t)w.n_events * nb, nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); q < bands; q += nwarps) {
+        const int n = w.band_counts[q];
+        if (!n) continue;
+        const int e = (int)(q / nb), o = w.band_offs[q], base = w.cand_base[e];
+        const unsigned hstart = (unsigned)w.hit_start[e];
+        const uint2 *list = w.band_cands + q * w.band_cap;
+        for (int k = lane; k < min(n, w.max_cand - o); k += 32) {
+            const uint2 v = list[k];
+            w.cand_list[base + o + k] = make_uint4(v.x, v.y, (unsigned)e, hstart);
+            if (records) {
+                uint4 *cd = reinterpret_cast<uint4 *>(w.cands + base + o + k);
+                cd[0] = make_uint4(v.x >> 16, v.x & 0xFFFFu, v.y, 0u);
+                cd[1] = make_uint4(0u, 0u, 0u, 0u);
+            }
+        }
+    }
+}
+
+// The first `limit` candidate records of all events to `out`, 16 bytes a thread.  When `stats_out` is
+// given, block 0 also copies the first event's counters there.
+__global__ void copy_candidates_kernel(Workspace w, hough_candidate *out, long long limit, DevStats *stats_out)
 {
     pdl_enter();
     static_assert(sizeof(DevStats) % 4 == 0, "the counters are copied as 32-bit words");
+    static_assert(sizeof(hough_candidate) == 32, "a record is two 16-byte vectors");
     if (stats_out && blockIdx.x == 0) {
         const uint32_t *src = reinterpret_cast<const uint32_t *>(w.stats);
         uint32_t *dst = reinterpret_cast<uint32_t *>(stats_out);
         for (int q = threadIdx.x; q < (int)(sizeof(DevStats) / 4); q += blockDim.x) dst[q] = src[q];
     }
-    const int total = w.cand_base[w.n_events];
-    const int n = rest ? total : (int)min((long long)total, limit);
-    for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < n; f += gridDim.x * blockDim.x) {
-        const int e = upper_index(w.cand_base, w.n_events, f);
-        const hough_candidate cd = w.cands[(int64_t)e * w.max_cand + (f - w.cand_base[e])];
-        if (f < limit) out[f] = cd;
-        else rest[f] = cd;
-    }
+    const long long n = 2 * min((long long)w.cand_base[w.n_events], limit);
+    const uint4 *src = reinterpret_cast<const uint4 *>(w.cands);
+    uint4 *dst = reinterpret_cast<uint4 *>(out);
+    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x)
+        dst[q] = src[q];
 }
 
 template <int TPB, bool GENERAL_ONLY, int CELL>
@@ -1625,33 +1542,19 @@ cudaError_t launch_band_peaks(const Axes &ax, const Workspace &w, const Tiling &
     return cudaGetLastError();
 }
 
-cudaError_t launch_compact(const Axes &ax, const Workspace &w, cudaStream_t stream)
+cudaError_t launch_compact(const Axes &ax, const Workspace &w, cudaStream_t stream, bool records)
 {
-    const int single = w.n_events == 1;
-    // about two CTAs per SM over all events (the copy of a dense event's tens of thousands of
-    // candidates is latency-bound in one CTA)
-    int dev = 0, sms = 152;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int parts = std::max(1, std::min(16, (2 * sms + w.n_events - 1) / w.n_events));
-    cudaError_t err = launch_chained(compact_kernel, dim3(w.n_events * parts), dim3(kCompactThreads), 0, stream, ax, w,
-                                     single, parts);
-    if (!err && !single) err = launch_chained(cand_scan_kernel, dim3(1), dim3(kCompactThreads), 0, stream, w);
-    return err;
-}
-
-cudaError_t launch_pack_candidates(const Axes &ax, const Workspace &w, hough_candidate *out, cudaStream_t stream,
-                                   long long limit, hough_candidate *rest, DevStats *stats_out, int blocks)
-{
-    (void)ax;
-    return launch_chained(pack_candidates_kernel, dim3(blocks), dim3(256), 0, stream, w, out, limit, rest, stats_out);
-}
-
-cudaError_t launch_peaks(const Axes &ax, const Workspace &w, const Tiling &t, cudaStream_t stream)
-{
-    cudaError_t err = launch_band_peaks(ax, w, t, stream);
+    cudaError_t err = launch_chained(band_scan_kernel, dim3(w.n_events), dim3(kCompactThreads), 0, stream, ax, w);
     if (err) return err;
-    return launch_compact(ax, w, stream);
+    const int64_t bands = (int64_t)w.n_events * n_bands(ax, w.band_rows);
+    const int blocks = (int)std::min<int64_t>((bands + 7) / 8, 1216);
+    return launch_chained(band_copy_kernel, dim3(blocks), dim3(256), 0, stream, ax, w, records ? 1 : 0);
+}
+
+cudaError_t launch_copy_candidates(const Workspace &w, hough_candidate *out, cudaStream_t stream, long long limit,
+                                   DevStats *stats_out, int blocks)
+{
+    return launch_chained(copy_candidates_kernel, dim3(blocks), dim3(256), 0, stream, w, out, limit, stats_out);
 }
 
 }  // namespace hough
