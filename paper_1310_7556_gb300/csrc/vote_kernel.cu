@@ -713,15 +713,14 @@ __global__ void __launch_bounds__(TPB, 1) gather_kernel(GatherParams p)
     // one 8-byte entry and a warp's loads cover consecutive entries
     constexpr int kCells = 8;
     uint16_t *M = w.M + (int64_t)e * ax.n_qpt * nphi;
-    constexpr int strip = kCells * 32;
-    const int per_row = (p.cols + strip - 1) / strip;
+    const int kc = min(kCells, p.cols >> 5);   // cells per lane (cols is a multiple of 64)
+    const int strip = kc * 32;
+    const int per_row = p.cols / strip;
     const int nstrips = nrows * per_row;
     const int lane = threadIdx.x & 31;
     for (int sidx = threadIdx.x >> 5; sidx < nstrips; sidx += TPB / 32) {
         const int rr = sidx / per_row;
-        const int s0 = (sidx - rr * per_row) * strip;      // the strip's first column of the tile
-        const int kc = min(kCells, (p.cols - s0) >> 5);    // cells per lane (cols is a multiple of 64)
-        const int jb = c0 + s0 + lane;
+        const int jb = c0 + (sidx - rr * per_row) * strip + lane;
         const unsigned vm = rowMask[rr];
         const int *rI = rowI + rr * 16;
         const unsigned *rG = rowG + rr * 16;
