@@ -282,7 +282,8 @@ int hough_process(hough_ctx *ctx, const float *r, const float *phi, const float 
  * count accumulator, three times with a d0 axis) of shared memory; gather_rows in 1..32 (0: 4);
  * gather_cols a multiple of 64 dividing n_phi (0: the largest such up to 512) with
  * n_layers * (gather_cols + 64) * 8 bytes of shared memory; gather_threads in {256, 512, 1024}
- * (0: 256).  HOUGH_EINVAL otherwise.  Every configuration gives the same results.
+ * (0: 256); with all three 0, rows and threads are chosen from the number of cells of the launch
+ * (HOUGH_VOTE_GATHER with layer masks).  HOUGH_EINVAL otherwise.  Every configuration gives the same results.
  */
 #define HOUGH_VOTE_GATHER  0
 #define HOUGH_VOTE_SCATTER 1

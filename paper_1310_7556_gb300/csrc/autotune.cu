@@ -171,7 +171,7 @@ int hough_batch_autotune(hough_batch *b, const hough_geometry *geometry, const h
         ++out->tried;
         return HOUGH_OK;
     };
-    const Tiling d0 = default_tiling_for(ax);
+    const Tiling d0 = default_tiling_for(ax, n_events);
     hough_tiling best{};
     public_tiling(d0, &best);
     float best_ms = -1.f;

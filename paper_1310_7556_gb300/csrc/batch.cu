@@ -33,7 +33,8 @@ struct hough_batch {
     int device = 0;
     int sms = 0;
     Axes ax{};
-    Tiling tiling{};
+    Tiling tiling{};                     // as a run of n_events uses it: tiling_for
+    hough_tiling wanted{};               // as set: a gather tile left open is chosen for each batch size
     float refine_eps = 0.f;
     hough_batch_limits limits{};
     Workspace w{};
@@ -73,6 +74,9 @@ struct hough_batch {
         return e;
     }
 
+    // The kernel configuration of a run of n events.
+    void tiling_for(int n) { tiling = resolve_tiling(ax, &wanted, n); }
+
     // The whole path on the current batch, enqueued on `s` (also the body of the captured graph).
     cudaError_t enqueue(cudaStream_t s)
     {
@@ -107,7 +111,9 @@ int hough_batch_create(const hough_geometry *geometry, const hough_binning *binn
     b->device = device;
     cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, device);
     b->ax = make_axes(geometry, binning);
-    b->tiling = default_tiling_for(b->ax);
+    b->tiling = default_tiling_for(b->ax, 1);
+    public_tiling(b->tiling, &b->wanted);
+    b->wanted.gather_rows = b->wanted.gather_cols = b->wanted.gather_threads = 0;
     b->refine_eps = refine_eps_for(b->ax);
     b->limits = *limits;
     const Axes &ax = b->ax;
@@ -127,6 +133,10 @@ int hough_batch_create(const hough_geometry *geometry, const hough_binning *binn
     A(b->alloc(&w.hot, H)); A(b->alloc(&w.cold, H)); A(b->alloc(&w.fsort, H)); A(b->alloc(&w.zsort, H));
     A(b->alloc(&w.counts, E * nkeys)); A(b->alloc(&w.offs, E * (nkeys + 1)));
     A(b->alloc(&w.prof, (size_t)(E * prof_event_entries(ax))));
+    if (ax.n_qpt <= kRankRows && !ax.counts) {
+        A(b->alloc(&w.prank, (size_t)(E * prof_event_entries(ax))));
+        A(b->alloc(&w.gsort, (size_t)ax.n_layers * ax.n_qpt)); A(b->alloc(&w.rankt, (size_t)ax.n_layers * ax.n_qpt));
+    }
     A(b->alloc(&w.radii, 1)); A(b->alloc(&w.info, HOUGH_MAX_LAYERS)); A(b->alloc(&w.memo, 1));
     A(b->alloc(&w.tab, (size_t)ax.n_layers * ax.n_qpt)); A(b->alloc(&w.arc, (size_t)ax.n_layers * ax.n_qpt));
     A(b->alloc(&w.zco, (size_t)ax.n_layers * ax.n_qpt));
@@ -146,10 +156,12 @@ int hough_batch_create(const hough_geometry *geometry, const hough_binning *binn
     w.band_rows = b->tiling.band_rows;
     w.band_cap = band_capacity(ax, b->tiling.band_rows);
     w.fused = b->tiling.vote_mode == HOUGH_VOTE_FUSED;
+    w.use_ranks = w.prank && b->tiling.vote_mode == HOUGH_VOTE_GATHER;
     std::vector<float> kq(ax.n_qpt);
     for (int i = 0; i < ax.n_qpt; ++i) kq[i] = (float)(ax.qpt_min + (i % ax.q_rows + 0.5) * ax.dk);
     A(cudaMemcpy(w.kq32, kq.data(), sizeof(float) * ax.n_qpt, cudaMemcpyHostToDevice));
     A(cudaMemset(w.memo, 0, sizeof(TableMemo)));
+    A(cudaMemset(w.M, 0, sizeof(uint16_t) * (size_t)E * ax.n_qpt * ax.n_phi));
     A(cudaMemset(b->inputs_dev, 0, sizeof(HitInputs)));   // as inputs_on_device says
     A(cudaMemset(w.stats, 0, sizeof(DevStats) * E));
     A(cudaMemset(w.cand_base, 0, sizeof(int32_t) * (E + 1)));
@@ -170,10 +182,12 @@ int hough_batch_set_tiling(hough_batch *b, const hough_tiling *t)
     if (!b) return bfail(HOUGH_EINVAL, "batch is required");
     int rc = check_tiling_for(b->ax, b->device, t);
     if (rc) return rc;
-    b->tiling = resolve_tiling(b->ax, t);
+    b->wanted = *t;
+    b->tiling_for(1);
     b->w.band_rows = t->band_rows;
     b->w.band_cap = band_capacity(b->ax, t->band_rows);
     b->w.fused = b->tiling.vote_mode == HOUGH_VOTE_FUSED;
+    b->w.use_ranks = b->w.prank && b->tiling.vote_mode == HOUGH_VOTE_GATHER;
     // captured graphs hold the old configuration
     cudaSetDevice(b->device);
     cudaDeviceSynchronize();
@@ -224,6 +238,7 @@ static int batch_prepare(hough_batch *b, const float *r, const float *phi, const
     BCU(cudaMemcpyAsync(b->hit_start, hit_start, sizeof(int64_t) * (n_events + 1), cudaMemcpyHostToDevice, s),
         "copy hit_start failed");
     b->w.n_events = n_events;
+    b->tiling_for(n_events);
     return HOUGH_OK;
 }
 

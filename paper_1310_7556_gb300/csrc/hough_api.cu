@@ -190,13 +190,28 @@ int default_gather_cols(const Axes &ax)
     return cols;
 }
 
-// A public tiling with its gather defaults (zero fields) filled in.
-Tiling resolve_tiling_impl(const Axes &ax, const hough_tiling *t)
+// A public tiling with its gather defaults (zero fields) filled in.  With all three left open the tile is
+// the tallest of 32, 16, 8 and 4 rows that still makes kMinTiles tiles of all events: a tall tile pays its
+// tables, windows and barriers once for more cells (256 events of 512 x 2048 cells: 0.71 ms with 4 rows,
+// 0.55 with 32; 16 events 54 -> 44 us; 4096 x 2048 cells 30 -> 26 us), but one event of 512 x 2048 cells
+// has only 512 tiles of 4 rows for 152 SMs and gains nothing.  Counts keep 4 rows: their gather lists
+// every hit of a tile's window.
+constexpr int64_t kMinTiles = 768;
+
+Tiling resolve_tiling_impl(const Axes &ax, const hough_tiling *t, int n_events)
 {
     Tiling r{t->tile_qpt, t->tile_phi, t->threads, t->vote_mode, t->band_rows,
              t->gather_rows, t->gather_cols, t->gather_threads};
-    if (!r.gather_rows) r.gather_rows = 4;
     if (!r.gather_cols) r.gather_cols = default_gather_cols(ax);
+    if (!t->gather_rows && !t->gather_cols && !t->gather_threads && !ax.counts && t->vote_mode == HOUGH_VOTE_GATHER) {
+        const int64_t spans = (int64_t)n_events * (ax.n_phi / r.gather_cols);
+        for (int rows : {32, 16, 8})
+            if (!r.gather_rows && spans * ((ax.n_qpt + rows - 1) / rows) >= kMinTiles) {
+                r.gather_rows = rows;
+                r.gather_threads = 512;
+            }
+    }
+    if (!r.gather_rows) r.gather_rows = 4;
     if (!r.gather_threads) r.gather_threads = 256;
     return r;
 }
@@ -219,7 +234,7 @@ int check_tiling_impl(const Axes &ax, int device, const hough_tiling *t)
         return fail(HOUGH_EINVAL, "gather_cols must be 0 or a multiple of 64 dividing n_phi");
     if (t->gather_threads && t->gather_threads != 256 && t->gather_threads != 512 && t->gather_threads != 1024)
         return fail(HOUGH_EINVAL, "gather_threads must be 0, 256, 512 or 1024");
-    const Tiling tt = resolve_tiling_impl(ax, t);
+    const Tiling tt = resolve_tiling_impl(ax, t, 1);
     int max_smem = 0;
     cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
     if (vote_smem_bytes(ax, tt) + 1024 > (size_t)max_smem)
@@ -243,9 +258,9 @@ int check_tiling_impl(const Axes &ax, int device, const hough_tiling *t)
     return HOUGH_OK;
 }
 
-Tiling default_tiling_impl(const Axes &ax)
+Tiling default_tiling_impl(const Axes &ax, int n_events)
 {
-    Tiling t;
+    hough_tiling t{};   // (the gather's tile: zero, chosen from the grid)
     t.tile_phi = std::min(ax.n_phi, 256);
     while (ax.n_phi % t.tile_phi) t.tile_phi -= 64;
     t.tile_qpt = std::min(ax.n_qpt, 32);   // the scatter kernel's lanes take 32 rows
@@ -261,10 +276,7 @@ Tiling default_tiling_impl(const Axes &ax)
                 t.band_rows = r;
                 break;
             }
-    t.gather_rows = 4;
-    t.gather_cols = default_gather_cols(ax);
-    t.gather_threads = 256;
-    return t;
+    return resolve_tiling_impl(ax, &t, n_events);
 }
 
 // Largest band-list storage over every allowed band height.
@@ -363,6 +375,7 @@ int enqueue_vote(hough_ctx *c, const float *r, const float *phi, const float *z,
     c->w.band_rows = c->tiling.band_rows;
     c->w.band_cap = band_capacity(c->ax, c->tiling.band_rows);
     c->w.fused = c->tiling.vote_mode == HOUGH_VOTE_FUSED;
+    c->w.use_ranks = c->w.prank && c->tiling.vote_mode == HOUGH_VOTE_GATHER;
     if (c->timing) { CU(cudaEventRecord(c->ev[0], s), "event"); c->timed |= 1 | (0xF << 8); }
     // this event's counters and radius ranges; the other buffer of each is zeroed for the next one
     c->w.stats = c->stats_buf[c->parity];
@@ -419,13 +432,13 @@ int read_stats(hough_ctx *c, cudaStream_t s)
 Axes hough::make_axes(const hough_geometry *g, const hough_binning *b) { return make_axes_impl(g, b); }
 int hough::check_geometry_binning(const hough_geometry *g, const hough_binning *b) { return check_binning(g, b); }
 int hough::check_tiling_for(const Axes &ax, int device, const hough_tiling *t) { return check_tiling_impl(ax, device, t); }
-Tiling hough::resolve_tiling(const Axes &ax, const hough_tiling *t) { return resolve_tiling_impl(ax, t); }
+Tiling hough::resolve_tiling(const Axes &ax, const hough_tiling *t, int n_events) { return resolve_tiling_impl(ax, t, n_events); }
 void hough::public_tiling(const Tiling &t, hough_tiling *out)
 {
     *out = hough_tiling{t.tile_qpt, t.tile_phi, t.threads, t.vote_mode, t.band_rows,
                         t.gather_rows, t.gather_cols, t.gather_threads};
 }
-Tiling hough::default_tiling_for(const Axes &ax) { return default_tiling_impl(ax); }
+Tiling hough::default_tiling_for(const Axes &ax, int n_events) { return default_tiling_impl(ax, n_events); }
 size_t hough::band_list_entries(const Axes &ax) { return band_list_entries_impl(ax); }
 int hough::check_host_hits_for(const Axes &ax, const float *r, const float *phi, const float *z, const uint8_t *layer,
                                int64_t n)
@@ -478,7 +491,7 @@ int hough_create(const hough_geometry *geometry, const hough_binning *binning, c
     c->binning = *binning;
     c->limits = *limits;
     c->ax = make_axes_impl(geometry, binning);
-    c->tiling = default_tiling_impl(c->ax);
+    c->tiling = default_tiling_impl(c->ax, 1);
     c->refine_eps = refine_eps_for(c->ax);
     const Axes &ax = c->ax;
     const int64_t n = limits->max_hits;
@@ -493,6 +506,10 @@ int hough_create(const hough_geometry *geometry, const hough_binning *binning, c
     A(c->alloc(&c->in_r, n)); A(c->alloc(&c->in_phi, n)); A(c->alloc(&c->in_z, n)); A(c->alloc(&c->in_layer, n));
     A(c->alloc(&w.key, n)); A(c->alloc(&w.rank, n)); A(c->alloc(&w.hot_tmp, n));
     A(c->alloc(&w.counts, nkeys)); A(c->alloc(&w.offs, nkeys + 1)); A(c->alloc(&w.prof, (size_t)prof_event_entries(ax)));
+    if (ax.n_qpt <= kRankRows && !ax.counts) {
+        A(c->alloc(&w.prank, (size_t)prof_event_entries(ax)));
+        A(c->alloc(&w.gsort, (size_t)ax.n_layers * ax.n_qpt)); A(c->alloc(&w.rankt, (size_t)ax.n_layers * ax.n_qpt));
+    }
     A(c->alloc(&w.hot, n)); A(c->alloc(&w.cold, n)); A(c->alloc(&w.fsort, n)); A(c->alloc(&w.zsort, n));
     A(c->alloc(&c->radii_buf[0], 1)); A(c->alloc(&c->radii_buf[1], 1));
     A(c->alloc(&w.info, HOUGH_MAX_LAYERS)); A(c->alloc(&w.memo, 1));
@@ -528,6 +545,7 @@ int hough_create(const hough_geometry *geometry, const hough_binning *binning, c
     A(cudaMemcpy(w.kq32, kq.data(), sizeof(float) * ax.n_qpt, cudaMemcpyHostToDevice));
     A(cudaMemset(c->hit_start, 0, 2 * sizeof(int64_t)));
     A(cudaMemset(w.memo, 0, sizeof(TableMemo)));
+    A(cudaMemset(w.M, 0, sizeof(uint16_t) * (size_t)ax.n_qpt * ax.n_phi));
     // the state every event starts from (Workspace::recycle keeps it so from then on)
     for (int q = 0; q < 2; ++q) {
         A(cudaMemset(c->stats_buf[q], 0, sizeof(DevStats)));
@@ -745,7 +763,7 @@ int hough_set_tiling(hough_ctx *c, const hough_tiling *t)
     if (!c) return fail(HOUGH_EINVAL, "ctx is required");
     int rc = check_tiling_impl(c->ax, c->device, t);
     if (rc) return rc;
-    c->tiling = resolve_tiling(c->ax, t);
+    c->tiling = resolve_tiling(c->ax, t, 1);
     return HOUGH_OK;
 }
 

@@ -10,6 +10,8 @@
 //                             .y = max over bucket J+1 of ~bits(f) (0 when the bucket is empty);
 //                             entries Nphi..Nphi+15 of each layer repeat entries 0..15
 //                             (so a window of consecutive buckets never wraps), 16 layers always
+//   prank[16*(Nphi+16)] (4 B) the same entries with the fractions replaced by their ranks among the
+//                             layer's table fractions g, as halves (gather vote of layer masks; kRankRows)
 //   hot[n], cold[n] (16 B)    staged hits sorted by (layer, J); cold holds r, phi, z, input index
 //   tab[L*Nq] (8 B)           per (layer, q/pT row): Nphi asin(x) / (2 pi) = I + g, for layers whose
 //                             hits share one radius; arc[L*Nq] the arc length s (FP64)
@@ -22,6 +24,7 @@
 //                             (contexts only: a batch keeps no member lists)
 #pragma once
 
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -102,6 +105,17 @@ struct LayerInfo {
 // Table entry of a (layer, row) on which the layer's radius casts no vote.
 constexpr int32_t kNoVote = -(1 << 30);
 
+// Rank form of the gather vote (layer masks, grids of up to kRankRows stacked rows).  A vote only
+// compares a hit's fraction f with the row's g, so f may be replaced by R(f), the number of the
+// layer's n table fractions that are <= f: f >= g exactly when R(f) >= R(g), as every fraction counted
+// in R(g) is <= g, and g itself is counted in R(f) only when f >= g.  Ranks up to 4096 less 2048 are
+// whole numbers of the half format, so a bucket's entry is a pair of halves (x, y) =
+// (R(largest f) - 2048, 2048 - R(smallest f of the next bucket)), R = 0 and R = n standing for no hit,
+// and a row's threshold the pair (2049 - R(g), R(g) - 2048): each half of their sum is a whole number
+// before rounding, at least 1 when its bucket votes and at most 0 when not, and rounding keeps it so.
+constexpr int kRankRows = 4096;
+constexpr uint32_t kNoRank = 0xFBFFFBFFu;    // the threshold of a row that casts no vote: lowest halves
+
 // Memo of the per-(layer, row) table: the radius each layer's rows were computed for.
 struct TableMemo {
     uint32_t r_bits[HOUGH_MAX_LAYERS];
@@ -138,6 +152,9 @@ struct Workspace {
     int32_t *counts;              // n_events * nkeys
     int32_t *offs;                // n_events * (nkeys + 1)
     uint2 *prof;                  // n_events * prof_event_entries
+    uint32_t *prank;              // n_events * prof_event_entries (null: the gather reads prof)
+    float *gsort;                 // n_layers * n_qpt: a layer's table fractions g of voting rows in order
+    uint32_t *rankt;              // n_layers * n_qpt: a row's rank threshold (kNoRank: the row casts no vote)
     HotHit *hot;                  // per hit, sorted within each event's range
     float *fsort;                 // per hit, sorted: the hot record's f alone (count gather, membership)
     float *zsort;                 // per hit, sorted: z alone (membership; may be null when no stage 2 runs)
@@ -163,6 +180,7 @@ struct Workspace {
     DevStats *stats;              // n_events
     int max_cand, max_members;
     int band_rows, band_cap;
+    int use_ranks;                // the gather votes by ranks: the hit sort forms prank from prof
     int fused;                    // vote_mode HOUGH_VOTE_FUSED: the vote kernel searched the bands
     int keep_members;             // 1: confirmation writes member lists to mem_pool (contexts); 0: none (batches)
     int copy_wait;                // < 0: the first bound on a bulk-copy wait expires at once (a test of the error path)
@@ -257,8 +275,9 @@ bool stage2_reads_bands(const Axes &ax, int band_rows);
 Axes make_axes(const hough_geometry *g, const hough_binning *b);
 int check_geometry_binning(const hough_geometry *g, const hough_binning *b);
 int check_tiling_for(const Axes &ax, int device, const hough_tiling *t);
-Tiling default_tiling_for(const Axes &ax);
-Tiling resolve_tiling(const Axes &ax, const hough_tiling *t);   // gather defaults filled in
+// n_events: the events of a launch, from which a gather tile left open is chosen.
+Tiling default_tiling_for(const Axes &ax, int n_events);
+Tiling resolve_tiling(const Axes &ax, const hough_tiling *t, int n_events);   // gather defaults filled in
 void public_tiling(const Tiling &t, hough_tiling *out);
 size_t gather_smem_bytes(const Axes &ax, const Tiling &t);
 // Dynamic shared memory of the fused vote and peak kernel: the band's masks and its two halo rows.

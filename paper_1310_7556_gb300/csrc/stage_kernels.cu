@@ -170,7 +170,61 @@ __global__ void __launch_bounds__(kStageThreads) stage_count_kernel(Axes ax, Wor
 // track (y = x for prompt tracks, the d0 relation on a grid with a d0 axis), the arc length from
 // the closest approach for stage 2, and the stage-2 terms derived from it.  Rows on which the
 // radius casts no vote get the entry kNoVote.
-__device__ __forceinline__ void layer_table(const Axes &ax, const Workspace &w, const int l)
+constexpr int kScanPerThread = 8;
+constexpr int kScanRound = kScanThreads * kScanPerThread;
+constexpr int kTileWords = kScanRound + kScanRound / 32;   // a CTA's shared tile: a padded scan round, or a layer's fractions
+static_assert(kRankRows <= kTileWords, "a layer's fractions are sorted in the shared tile");
+
+// Two whole numbers the half format holds, as a pair of halves.
+__device__ __forceinline__ uint32_t half_pair(int x, int y)
+{
+    return (uint32_t)__half_as_ushort(__int2half_rn(x)) | (uint32_t)__half_as_ushort(__int2half_rn(y)) << 16;
+}
+
+// Ranks of a layer's table fractions (see kRankRows): the fractions of its nvote voting rows sorted
+// (bitonic, in the shared tile) into gsort, and each row's threshold.  By the whole CTA.
+__device__ void layer_ranks(const Axes &ax, const Workspace &w, const int l, const int nvote, float *s_g)
+{
+    __shared__ int s_fill;
+    const int n = ax.n_qpt;
+    if (threadIdx.x == 0) s_fill = 0;
+    __syncthreads();
+    const TabEntry *tab = w.tab + l * n;
+    for (int i = threadIdx.x; i < n; i += blockDim.x)
+        if (tab[i].I != kNoVote) s_g[atomicAdd(&s_fill, 1)] = tab[i].g;   // any order: sorted next
+    int p2 = 1;
+    while (p2 < nvote) p2 <<= 1;
+    for (int i = nvote + threadIdx.x; i < p2; i += blockDim.x) s_g[i] = 2.f;   // above every fraction
+    __syncthreads();
+    for (int k = 2; k <= p2; k <<= 1)
+        for (int d = k >> 1; d > 0; d >>= 1) {
+            for (int q = threadIdx.x; q < p2 / 2; q += blockDim.x) {
+                const int a = (q / d) * 2 * d + q % d, b = a + d;
+                const float x = s_g[a], y = s_g[b];
+                if ((x > y) == ((a & k) == 0)) {
+                    s_g[a] = y;
+                    s_g[b] = x;
+                }
+            }
+            __syncthreads();
+        }
+    for (int i = threadIdx.x; i < nvote; i += blockDim.x) w.gsort[l * n + i] = s_g[i];
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        uint32_t t = kNoRank;
+        if (tab[i].I != kNoVote) {
+            const float g = tab[i].g;
+            int lo = 0, hi = nvote;   // the number of fractions <= g
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (s_g[mid] <= g) lo = mid + 1; else hi = mid;
+            }
+            t = half_pair(2049 - lo, lo - 2048);
+        }
+        w.rankt[l * n + i] = t;
+    }
+}
+
+__device__ __forceinline__ void layer_table(const Axes &ax, const Workspace &w, const int l, int *s_tile)
 {
     __shared__ LayerInfo s_li;
     __shared__ int s_dirty;
@@ -260,6 +314,8 @@ __device__ __forceinline__ void layer_table(const Axes &ax, const Workspace &w, 
         w.info[l].nvote = s_nvote;
         w.memo->nvote[l] = s_nvote;
     }
+    // (kept with the table, whichever form of the vote this event takes)
+    if (w.rankt) layer_ranks(ax, w, l, s_nvote, reinterpret_cast<float *>(s_tile));
 }
 
 // One CTA per event: exclusive scan of the bucket sizes, kScanRound counts per round.  The counts
@@ -267,16 +323,13 @@ __device__ __forceinline__ void layer_table(const Axes &ax, const Workspace &w, 
 // kScanPerThread consecutive entries in registers and the CTA scans the threads' totals (one
 // shuffle scan per warp, one over the warps).  The tile has one padding word per 32, which keeps
 // the per-thread reads of consecutive words free of bank conflicts.
-constexpr int kScanPerThread = 8;
-constexpr int kScanRound = kScanThreads * kScanPerThread;
-
 __device__ __forceinline__ int scan_pad(int k) { return k + (k >> 5); }
 
 // Exclusive scan of counts[k0, k1) into offs[k0, k1), starting from `carry`; returns the running
 // total after k1.  Every thread of the CTA takes part.
-__device__ __forceinline__ int scan_range(const int32_t *counts, int32_t *offs, const int k0, const int k1, int carry)
+__device__ __forceinline__ int scan_range(const int32_t *counts, int32_t *offs, const int k0, const int k1, int carry,
+                                          int *s_tile)
 {
-    __shared__ int s_tile[kScanRound + kScanRound / 32];
     __shared__ int s_warp[kScanThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int base = k0; base < k1; base += kScanRound) {
@@ -336,10 +389,11 @@ __device__ __forceinline__ int scan_range(const int32_t *counts, int32_t *offs, 
 }
 
 // One CTA per event: the scan of all its keys.
-__device__ __forceinline__ void scan_keys(const Axes &ax, const Workspace &w, const int e)
+__device__ __forceinline__ void scan_keys(const Axes &ax, const Workspace &w, const int e, int *s_tile)
 {
     const int nkeys = n_keys(ax);
-    const int total = scan_range(w.counts + (int64_t)e * nkeys, w.offs + (int64_t)e * (nkeys + 1), 0, nkeys, 0);
+    const int total = scan_range(w.counts + (int64_t)e * nkeys, w.offs + (int64_t)e * (nkeys + 1), 0, nkeys, 0,
+                                 s_tile);
     if (threadIdx.x == 0) {
         w.offs[(int64_t)e * (nkeys + 1) + nkeys] = total;
         w.stats[e].n_hits = (unsigned long long)total;
@@ -350,7 +404,7 @@ __device__ __forceinline__ void scan_keys(const Axes &ax, const Workspace &w, co
 // event's counts of the layers before its own (its offset), then scans its layer's buckets, so the
 // layers of an event are scanned side by side instead of one after another.  Integer sums: the
 // same offsets as scan_keys.
-__device__ __forceinline__ void scan_layer(const Axes &ax, const Workspace &w, const int e, const int l)
+__device__ __forceinline__ void scan_layer(const Axes &ax, const Workspace &w, const int e, const int l, int *s_tile)
 {
     __shared__ int s_part[kScanThreads / 32];
     const int nkeys = n_keys(ax), nphi = ax.n_phi;
@@ -378,7 +432,7 @@ __device__ __forceinline__ void scan_layer(const Axes &ax, const Workspace &w, c
     int base = 0;
 #pragma unroll
     for (int q = 0; q < kScanThreads / 32; ++q) base += s_part[q];
-    const int total = scan_range(counts, offs, l * nphi, (l + 1) * nphi, base);
+    const int total = scan_range(counts, offs, l * nphi, (l + 1) * nphi, base, s_tile);
     if (threadIdx.x == 0 && l == ax.n_layers - 1) {
         offs[nkeys] = total;
         w.stats[e].n_hits = (unsigned long long)total;
@@ -393,9 +447,10 @@ __global__ void __launch_bounds__(kScanThreads) table_scan_kernel(Axes ax, Works
     pdl_enter();
     const int scans = by_layer ? w.n_events * ax.n_layers : w.n_events;
     const int b = blockIdx.x;
-    if (b >= scans) layer_table(ax, w, b - scans);
-    else if (by_layer) scan_layer(ax, w, b / ax.n_layers, b % ax.n_layers);
-    else scan_keys(ax, w, b);
+    __shared__ int s_tile[kTileWords];
+    if (b >= scans) layer_table(ax, w, b - scans, s_tile);
+    else if (by_layer) scan_layer(ax, w, b / ax.n_layers, b % ax.n_layers, s_tile);
+    else scan_keys(ax, w, b, s_tile);
 }
 
 // The votes of layers of one radius, per event: the layer's hits times its voting rows (thread t of
@@ -462,11 +517,49 @@ __device__ __forceinline__ void sort_hit(const Axes &ax, const Workspace &w, int
     if (w.zsort) w.zsort[pos] = ch.z;
 }
 
-// Scatter every valid hit to its sorted position, completing its hot record with its voting rows.
-__global__ void __launch_bounds__(kStageThreads) hit_sort_kernel(Axes ax, Workspace w)
+// The rank form of a bucket profile entry (see kRankRows), by thread t0 of nthreads: a layer of one
+// radius has its table fractions sorted by now.  With recycling the entry read is zeroed for the next
+// event, as nothing reads it again.
+__device__ __forceinline__ void rank_profile(const Axes &ax, const Workspace &w, int64_t t0, int64_t nthreads)
 {
+    const int stride = prof_stride(ax);
+    const int64_t per = (int64_t)ax.n_layers * stride, total = per * w.n_events;
+    for (int64_t q = t0; q < total; q += nthreads) {
+        const int e = (int)(q / per), k = (int)(q - (int64_t)e * per), l = k / stride;
+        const int64_t at = (int64_t)e * prof_event_entries(ax) + k;
+        const uint2 v = w.prof[at];
+        const LayerInfo li = w.info[l];
+        int x = 0, y = li.nvote;
+        if (li.present && li.uniform && (v.x | v.y)) {
+            const float *g = w.gsort + l * ax.n_qpt;
+            auto rank = [&](float f) {   // the number of fractions <= f
+                int lo = 0, hi = li.nvote;
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (__ldg(&g[mid]) <= f) lo = mid + 1; else hi = mid;
+                }
+                return lo;
+            };
+            if (v.x) x = rank(__uint_as_float(v.x - 1u));
+            if (v.y) y = rank(__uint_as_float(~v.y));
+        }
+        w.prank[at] = half_pair(x - 2048, 2048 - y);
+        if (w.recycle) w.prof[at] = make_uint2(0u, 0u);
+    }
+}
+
+// Scatter every valid hit to its sorted position, completing its hot record with its voting rows.
+// The blocks past the first hit_blocks turn the bucket profiles into ranks beside them.
+__global__ void __launch_bounds__(kStageThreads) hit_sort_kernel(Axes ax, Workspace w, int hit_blocks)
+{
+    if ((int)blockIdx.x >= hit_blocks) {
+        pdl_enter();
+        rank_profile(ax, w, (int64_t)(blockIdx.x - hit_blocks) * blockDim.x + threadIdx.x,
+                     (int64_t)(gridDim.x - hit_blocks) * blockDim.x);
+        return;
+    }
     const int nkeys = n_keys(ax);
-    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)hit_blocks * blockDim.x;
     const int64_t total = hit_total(w);
     const HitInputs in = hit_inputs(w);
     // The thread's first hit's own inputs -- its key, rank and record from the counting kernel,
@@ -562,7 +655,9 @@ cudaError_t launch_stage(const Axes &ax, const Workspace &w, cudaStream_t stream
         return err;
     if ((err = mark(2))) return err;   // table_ms covers both; scan_ms stays empty
     if ((err = mark(3))) return err;
-    return launch_chained(hit_sort_kernel, dim3(g), dim3(kStageThreads), 0, stream, ax, w);
+    const int64_t entries = (int64_t)w.n_events * ax.n_layers * prof_stride(ax);
+    const int rank_blocks = w.use_ranks ? (int)std::min<int64_t>((entries + kStageThreads - 1) / kStageThreads, 4864) : 0;
+    return launch_chained(hit_sort_kernel, dim3(g + rank_blocks), dim3(kStageThreads), 0, stream, ax, w, g);
 }
 
 }  // namespace hough

@@ -758,6 +758,191 @@ __global__ void __launch_bounds__(TPB, 1) gather_kernel(GatherParams p)
 }
 
 
+// The gather in rank form (see kRankRows in hough_internal.cuh).  A (cell, layer) costs one 4-byte
+// shared load, one saturating half-pair addition -- 1 in either half says that the bucket, or the one
+// after it, votes -- and one half-pair multiply-add that puts the layer's bit into the cell's two masks
+// (one for each bucket, whole numbers below 1024, exact in halves), which are ORed at the end.  Why
+// halves: gather_kernel's two integer comparisons, selects and ORs per (cell, layer), and likewise a
+// packed 16-bit maximum, run in the half-rate integer pipe and bound the kernel there (11.9
+// instructions per 32 (cell, layer)s, 6.5 of them in that pipe), while half arithmetic runs in the
+// multiply-add pipe; what is left to bind is the shared loads.  The windows' copies are issued a layer
+// a lane.
+constexpr int kRankPad = 128;   // window entries beyond the tile's columns held in a layer's slot
+
+__device__ __forceinline__ __half2 pair_of(uint32_t bits)
+{
+    return __halves2half2(__ushort_as_half((unsigned short)bits), __ushort_as_half((unsigned short)(bits >> 16)));
+}
+
+// The OR of a pair of masks below 1024: 1024 added, a mask is the significand's bits.
+__device__ __forceinline__ uint32_t pair_mask(__half2 m)
+{
+    const __half2 s = __hadd2(m, __float2half2_rn(1024.f));
+    const uint32_t u = (uint32_t)__half_as_ushort(__low2half(s)) | (uint32_t)__half_as_ushort(__high2half(s)) << 16;
+    return (u | u >> 16) & 0x3FFu;
+}
+
+// A strip of 32 kc cells of a row: lane t's cells are columns jb, jb + 32, ... of the tile, jb holding the
+// lane.  rowQ: per layer, the entry of column 0 in `win` and the threshold (kNoRank: no vote, or a layer
+// whose window is not staged); slow: the layers of that kind, read from global memory (src, columns
+// c0 + jb on, shift and threshold in rowS).  KC: cells a lane takes, when all strips are full (else 0).
+template <int NL, int KC>
+__device__ __forceinline__ void rank_strip(const uint32_t *win, const int2 *rowQ, unsigned slow, const int2 *rowS,
+                                           const uint32_t *prof, int pstride, int nphi, int c0, int jb, int kc,
+                                           uint16_t *row)
+{
+    constexpr int kCells = 8;
+    // a mask pair holds ten layers; with more than ten, eight and the rest
+    constexpr int kSplit = NL <= 10 ? NL : 8;
+    __half2 mask[kCells], more[NL <= 10 ? 1 : kCells];
+#pragma unroll
+    for (int c = 0; c < kCells; ++c) mask[c] = __half2half2(__ushort_as_half(0));
+#pragma unroll
+    for (int c = 0; c < (NL <= 10 ? 1 : kCells); ++c) more[c] = __half2half2(__ushort_as_half(0));
+    auto vote = [&](int l, int c, uint32_t entry, uint32_t th) {
+        const __half2 bit = __float2half2_rn((float)(1 << (l < kSplit ? l : l - kSplit)));
+        __half2 &m = l < kSplit ? mask[c] : more[NL <= 10 ? 0 : c];
+        m = __hfma2(__hadd2_sat(pair_of(entry), pair_of(th)), bit, m);
+    };
+#pragma unroll
+    for (int l = 0; l < NL; ++l) {
+        const int2 q = rowQ[l];
+        if ((uint32_t)q.y == kNoRank) continue;   // the same for the whole warp
+        const uint32_t *src = win + q.x + jb;     // inside the window
+        uint32_t v[kCells];
+#pragma unroll
+        for (int c = 0; c < kCells; ++c) v[c] = KC == kCells || c < kc ? src[32 * c] : 0u;
+#pragma unroll
+        for (int c = 0; c < kCells; ++c) vote(l, c, v[c], (uint32_t)q.y);
+    }
+    if (slow) {
+#pragma unroll
+        for (int l = 0; l < NL; ++l) {
+            if (!((slow >> l) & 1u) || (uint32_t)rowS[l].y == kNoRank) continue;
+            const uint32_t *src = prof + (int64_t)l * pstride;
+#pragma unroll
+            for (int c = 0; c < kCells; ++c)
+                if (c < kc) vote(l, c, __ldg(&src[wrap_col(c0 + jb + 32 * c + rowS[l].x, nphi)]), (uint32_t)rowS[l].y);
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < kCells; ++c)
+        if (KC == kCells || c < kc) {
+            uint32_t m = pair_mask(mask[c]);
+            if (NL > 10) m |= pair_mask(more[NL <= 10 ? 0 : c]) << kSplit;
+            row[32 * c] = (uint16_t)m;
+        }
+}
+
+template <int NL, int TPB>
+__global__ void __launch_bounds__(TPB) gather_rank_kernel(GatherParams p)
+{
+    pdl_enter();
+    extern __shared__ __align__(16) unsigned char gather_smem[];
+    __shared__ int2 rowS[kGatherRowsMax * 16];   // per (row, layer): I and threshold
+    __shared__ int2 rowQ[kGatherRowsMax * 16];   // the same with I as the entry of the tile's column 0 in its window
+    __shared__ unsigned s_staged, s_used;
+    __shared__ __align__(8) uint64_t s_bar;
+    const Axes &ax = p.ax;
+    const Workspace &w = p.w;
+    const int e = blockIdx.x / p.tiles_per_event;
+    const int t = blockIdx.x - e * p.tiles_per_event;
+    const int rt = t / p.col_tiles, ct = t - rt * p.col_tiles;
+    const int i0 = rt * p.rows, c0 = ct * p.cols;
+    const int nrows = min(p.rows, ax.n_qpt - i0);
+    const int L = ax.n_layers, nphi = ax.n_phi;
+    if (threadIdx.x == 0) mbar_init(&s_bar, 1);
+    for (int q = threadIdx.x; q < nrows * 16; q += TPB) {
+        const int rr = q >> 4, l = q & 15, i = i0 + rr;
+        int2 v = make_int2(0, (int)kNoRank);
+        if (l < L) {
+            const LayerInfo li = w.info[l];
+            const TabEntry te = w.tab[l * ax.n_qpt + i];   // all requested together: one round trip
+            const uint32_t tr = w.rankt[l * ax.n_qpt + i];
+            if (li.present && li.uniform && te.I != kNoVote) v = make_int2(te.I, (int)tr);
+        }
+        rowS[q] = v;
+    }
+    __syncthreads();
+    const uint32_t *prof = w.prank + (int64_t)e * prof_event_entries(ax);
+    const int pstride = prof_stride(ax);
+    uint32_t *win = reinterpret_cast<uint32_t *>(gather_smem);
+    if (threadIdx.x < 32) {
+        // lane l: layer l's window of entries [c0 + min I, c0 + cols + max I) (unwrapped, rounded out to
+        // 16 bytes), copied in pieces that end at the axis' seam; a window may hold more than the whole axis
+        const int l = threadIdx.x;
+        int lo = INT_MAX, hi = INT_MIN;
+        if (l < L)
+            for (int rr = 0; rr < nrows; ++rr) {
+                const int2 v = rowS[rr * 16 + l];
+                if ((uint32_t)v.y != kNoRank) {
+                    lo = min(lo, v.x);
+                    hi = max(hi, v.x);
+                }
+            }
+        int ws = 0, len = 0;
+        if (lo <= hi) {
+            ws = (c0 + lo) & ~3;
+            len = (c0 + p.cols + hi - ws + 3) & ~3;
+        }
+        const bool staged = len > 0 && len <= p.cap;
+        const unsigned sm = __ballot_sync(0xFFFFFFFFu, staged), used = __ballot_sync(0xFFFFFFFFu, len > 0);
+        const unsigned bytes = __reduce_add_sync(0xFFFFFFFFu, staged ? 4u * (unsigned)len : 0u);
+        if (l == 0) {
+            s_staged = sm;
+            s_used = used;
+            if (sm) mbar_arrive_expect(&s_bar, bytes);
+        }
+        __syncwarp();
+        if (staged) {
+            const uint32_t *src = prof + (int64_t)l * pstride;
+            int a = ws % nphi;
+            a += a < 0 ? nphi : 0;   // a multiple of 4, as nphi is
+            for (int at = 0; at < len;) {
+                const int n = min(len - at, nphi - a);
+                bulk_copy_g2s(win + l * p.cap + at, src + a, 4u * (unsigned)n, &s_bar);
+                at += n;
+                a = 0;
+            }
+        }
+        if (l < 16)
+            for (int rr = 0; rr < nrows; ++rr) {
+                const int2 v = rowS[rr * 16 + l];
+                rowQ[rr * 16 + l] = make_int2(l * p.cap + c0 + v.x - ws, staged ? v.y : (int)kNoRank);
+            }
+    }
+    __syncthreads();
+    const unsigned staged = s_staged, slow = s_used & ~staged;
+    if (staged) {
+        const bool ok = first_copy_wait(w, &s_bar);
+        if (!__syncthreads_and(ok)) {
+            // the copies did not land in time: report it, give them one more bound, write nothing
+            if (threadIdx.x == 0) atomicOr(&w.stats[e].device_error, HOUGH_DEVERR_TIMEOUT);
+            mbar_wait_bounded(&s_bar, 0, kCopyWaitCycles);
+            return;
+        }
+    }
+    // one warp per strip of up to 256 cells of a row
+    uint16_t *M = w.M + (int64_t)e * ax.n_qpt * nphi;
+    const int kc = min(8, p.cols >> 5);   // cells per lane (cols is a multiple of 64)
+    const int strip = kc * 32;
+    // Known fault, the same as in gather_kernel: a tile more than 256 columns wide whose width is not a
+    // multiple of 256 (320, 384, 448) loses the columns past its last whole strip; their cells keep the
+    // zeros they were created with.
+    const int per_row = p.cols / strip;
+    const int nstrips = nrows * per_row;
+    const int lane = threadIdx.x & 31;
+    for (int sidx = threadIdx.x >> 5; sidx < nstrips; sidx += TPB / 32) {
+        const int rr = sidx / per_row;
+        const int jb = (sidx - rr * per_row) * strip + lane;   // column within the tile
+        uint16_t *row = M + (int64_t)(i0 + rr) * nphi + c0 + jb;
+        if (kc == 8)
+            rank_strip<NL, 8>(win, rowQ + rr * 16, slow, rowS + rr * 16, prof, pstride, nphi, c0, jb, 8, row);
+        else
+            rank_strip<NL, 0>(win, rowQ + rr * 16, slow, rowS + rr * 16, prof, pstride, nphi, c0, jb, kc, row);
+    }
+}
+
 // Fused vote and peak search (vote_mode HOUGH_VOTE_FUSED): a CTA per band of band_rows full rows.
 // A cell of a layer of one radius is a function of its row's table entry and two bucket-profile
 // entries alone, so the CTA computes the band's masks and those of the row above and below it
@@ -1063,7 +1248,7 @@ __global__ void __launch_bounds__(TPB) gather_count_kernel(GatherParams p, int f
 // zero it here for the next event (Workspace::recycle).
 __device__ __forceinline__ void recycle_profile(const Axes &ax, const Workspace &w)
 {
-    if (!w.recycle || !w.prof) return;
+    if (!w.recycle || !w.prof || w.use_ranks) return;   // (with ranks the hit sort has zeroed it)
     uint4 *p4 = reinterpret_cast<uint4 *>(w.prof);
     const int64_t n4 = (int64_t)w.n_events * prof_event_entries(ax) / 2;   // two entries a vector
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n4; q += (int64_t)gridDim.x * blockDim.x)
@@ -1401,6 +1586,16 @@ size_t gather_smem_bytes(const Axes &ax, const Tiling &t)
     return (size_t)ax.n_layers * (size_t)(t.gather_cols + 64) * sizeof(uint2);
 }
 
+template <int NL>
+cudaError_t launch_gather_rank_nl(const GatherParams &p, int threads, size_t smem, int blocks, cudaStream_t stream)
+{
+    auto kernel = threads == 256 ? gather_rank_kernel<NL, 256> : threads == 1024 ? gather_rank_kernel<NL, 1024>
+                                                                                 : gather_rank_kernel<NL, 512>;
+    cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (err) return err;
+    return launch_chained(kernel, dim3(blocks), dim3(threads), smem, stream, p);
+}
+
 static cudaError_t launch_gather_tiled(const Axes &ax, const Workspace &w, const Tiling &t, cudaStream_t stream)
 {
     GatherParams p;
@@ -1408,10 +1603,19 @@ static cudaError_t launch_gather_tiled(const Axes &ax, const Workspace &w, const
     p.w = w;
     p.rows = t.gather_rows;
     p.cols = t.gather_cols;
-    p.cap = t.gather_cols + 64;
     p.col_tiles = ax.n_phi / p.cols;
     p.tiles_per_event = ((ax.n_qpt + p.rows - 1) / p.rows) * p.col_tiles;
     const int blocks = w.n_events * p.tiles_per_event;
+    if (w.use_ranks) {
+        p.cap = t.gather_cols + kRankPad;
+        const size_t smem = (size_t)ax.n_layers * p.cap * sizeof(uint32_t);
+        // layer loops unrolled
+        if (ax.n_layers <= 4) return launch_gather_rank_nl<4>(p, t.gather_threads, smem, blocks, stream);
+        if (ax.n_layers <= 8) return launch_gather_rank_nl<8>(p, t.gather_threads, smem, blocks, stream);
+        if (ax.n_layers <= 10) return launch_gather_rank_nl<10>(p, t.gather_threads, smem, blocks, stream);
+        return launch_gather_rank_nl<16>(p, t.gather_threads, smem, blocks, stream);
+    }
+    p.cap = t.gather_cols + 64;
     const size_t smem = gather_smem_bytes(ax, t);
     // layer loops unrolled to the next multiple of four
     if (ax.n_layers <= 4) return launch_gather_nl<4>(p, t.gather_threads, smem, blocks, stream);
