@@ -502,12 +502,14 @@ __device__ __forceinline__ void row_range(const Axes &ax, double c, int *lo_out,
 {
     const int n = ax.n_qpt;
     auto valid = [&](int i) { return fabs(__dmul_rn(c, qpt_centre(ax, i))) <= 1.0; };
-    double klim = 1.0 / c;
-    double flo = ceil((-klim - ax.qpt_min) / ax.dk - 0.5);
-    double fhi = floor((klim - ax.qpt_min) / ax.dk - 0.5);
-    int lo = (int)fmin(fmax(flo, 0.0), (double)(n - 1));
-    int hi = (int)fmin(fmax(fhi, 0.0), (double)(n - 1));
-    // the estimates sit within a row of the true edges; settle them with the exact predicate
+    // (single precision is enough for estimates: three FP64 divisions a hit took most of the hit sort's
+    // time on a detector whose every hit has a radius of its own)
+    const float klim = __fdividef(1.f, (float)c), q0 = (float)ax.qpt_min, rdk = __fdividef(1.f, (float)ax.dk);
+    const float flo = ceilf((-klim - q0) * rdk - 0.5f);
+    const float fhi = floorf((klim - q0) * rdk - 0.5f);
+    int lo = (int)fminf(fmaxf(flo, 0.f), (float)(n - 1));
+    int hi = (int)fminf(fmaxf(fhi, 0.f), (float)(n - 1));
+    // the estimates sit within a row or two of the true edges; settle them with the exact predicate
     while (lo > 0 && valid(lo - 1)) --lo;
     while (lo < n && !valid(lo)) ++lo;
     if (lo >= n) { *lo_out = 1; *hi_out = 0; return; }

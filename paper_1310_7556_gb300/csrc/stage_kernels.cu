@@ -482,7 +482,8 @@ __device__ __forceinline__ void recycle_counts(const Axes &ax, const Workspace &
 // Valid hit h (input index; event start `start`) to its sorted position pos: its f, hot record hh
 // completed with its voting rows, cold record (r, phi, z) and z.
 __device__ __forceinline__ void sort_hit(const Axes &ax, const Workspace &w, int64_t h, int e, int64_t start,
-                                         int64_t pos, HotHit hh, float rr, float ph, float zz)
+                                         int64_t pos, HotHit hh, float rr, float ph, float zz, int e0,
+                                         unsigned *s_votes)
 {
     if (w.fsort) w.fsort[pos] = hh.f;
     const int l = (hh.jl >> 16) & 0xF;
@@ -502,8 +503,10 @@ __device__ __forceinline__ void sort_hit(const Axes &ax, const Workspace &w, int
         if (nv) atomicAdd(&w.stats[e].votes_by_layer[l], nv);
     } else if (!li.uniform) {
         row_range(ax, sagitta_coef(ax, (double)rr), &lo, &hi);
-        if (hi >= lo)
-            atomicAdd(&w.stats[e].votes_by_layer[l], (unsigned long long)(hi - lo + 1));
+        // (counted per CTA first: a 64-bit atomic per hit on a handful of counters took 20 us of the 100k-hit
+        // event's sort; a CTA's hits are almost all of one event)
+        if (hi >= lo && e == e0) atomicAdd(&s_votes[l], (unsigned)(hi - lo + 1));
+        else if (hi >= lo) atomicAdd(&w.stats[e].votes_by_layer[l], (unsigned long long)(hi - lo + 1));
     }
     if (hi < lo) { lo = 1; hi = 0; }
     hh.rows = (uint32_t)lo | ((uint32_t)hi << 16);
@@ -576,7 +579,12 @@ __global__ void __launch_bounds__(kStageThreads) hit_sort_kernel(Axes ax, Worksp
         ph = in.phi[t0];
         zz = in.z[t0];
     }
+    __shared__ unsigned s_votes[HOUGH_MAX_LAYERS];
+    if (threadIdx.x < HOUGH_MAX_LAYERS) s_votes[threadIdx.x] = 0u;
     pdl_enter();
+    __syncthreads();
+    const int64_t first = (int64_t)blockIdx.x * blockDim.x;
+    const int e0 = first < total ? event_of(w.hit_start, w.n_events, first) : 0;
     // this thread's first (event, layer) pair of the one-radius vote counts: its inputs requested
     // now, counted after the hits, so the loads overlap the hits' own
     const int64_t npairs = (int64_t)w.n_events * ax.n_layers;
@@ -602,12 +610,15 @@ __global__ void __launch_bounds__(kStageThreads) hit_sort_kernel(Axes ax, Worksp
         }
         const int e = event_of(w.hit_start, w.n_events, h);
         const int64_t start = w.hit_start[e];
-        if (k >= 0) sort_hit(ax, w, h, e, start, start + w.offs[(int64_t)e * (nkeys + 1) + k] + rank, hh, rr, ph, zz);
+        if (k >= 0) sort_hit(ax, w, h, e, start, start + w.offs[(int64_t)e * (nkeys + 1) + k] + rank, hh, rr, ph, zz, e0, s_votes);
     }
     if (t0 < npairs && tli.present && tli.uniform && tli.nvote > 0 && tn)
         atomicAdd(&w.stats[te].votes_by_layer[tl], (unsigned long long)tn * (unsigned long long)tli.nvote);
     count_table_votes(ax, w, t0 + nt, nt, [&](int e, int k) { return w.offs[(int64_t)e * (nkeys + 1) + k]; });
     if (w.recycle) recycle_counts(ax, w, t0, nt);
+    __syncthreads();
+    if (threadIdx.x < HOUGH_MAX_LAYERS && s_votes[threadIdx.x])
+        atomicAdd(&w.stats[e0].votes_by_layer[threadIdx.x], (unsigned long long)s_votes[threadIdx.x]);
 }
 
 int grid_for(int64_t n, int threads)

@@ -38,6 +38,7 @@
 #include <algorithm>
 #include <atomic>
 #include <climits>
+#include <type_traits>
 
 #include "hough_internal.cuh"
 
@@ -158,22 +159,16 @@ __device__ __forceinline__ void tile_vote_if(uint32_t *rowp, int stride, int jt,
     else atomicOr(&rowp[(jc >> 1) * stride], in ? lbit << ((jc & 1) << 4) : 0u);
 }
 
-template <int TPB, bool GENERAL_ONLY, int CELL>
+template <int TPB, int CELL>
 __global__ void __launch_bounds__(TPB) scatter_kernel(VoteParams p)
 {
     constexpr bool COUNTS = CELL == 2;
-    // After the gather (GENERAL_ONLY) this kernel reads nothing its predecessor writes until its
-    // flush ORs its tile into the gathered accumulator: the layer records, tables, bucket offsets
-    // and sorted hits come from kernels that finished before the gather could launch.  So it checks
-    // for layers of several radii and casts their votes first, and waits for the gather only before
-    // the flush (or before returning with nothing to do), which keeps its completion behind the
-    // gather's.  Voting every layer, it follows the hit sort and waits at once.
-    if (!GENERAL_ONLY) pdl_enter();
+    pdl_enter();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_start[kMaxRanges], s_off[kMaxRanges];
     __shared__ int s_pre[kMaxRanges + 1];
     __shared__ unsigned long long s_refined;
-    __shared__ unsigned s_umask, s_gmask;
+    __shared__ unsigned s_umask;
     __shared__ unsigned s_fast;   // table layers whose spread of I fits the tile's margins
 
     const Axes &ax = p.ax;
@@ -209,18 +204,12 @@ __global__ void __launch_bounds__(TPB) scatter_kernel(VoteParams p)
         unsigned u, g;
         layer_masks(p.w, L, &u, &g);
         if (threadIdx.x == 0) {
-            s_umask = GENERAL_ONLY ? ~g : u;   // layers this kernel treats with the table
-            s_gmask = g;
+            s_umask = u;   // layers treated with the table
             s_refined = 0ull;
             s_fast = 0u;
         }
     }
     __syncthreads();
-    // in gather mode there is nothing to do unless some layer has hits at several radii
-    if (GENERAL_ONLY && s_gmask == 0u) {
-        pdl_enter();
-        return;
-    }
     const unsigned umask = s_umask;
 
     // clear the tile; stage this slab's table rows and FP32 q/pT centres
@@ -231,7 +220,7 @@ __global__ void __launch_bounds__(TPB) scatter_kernel(VoteParams p)
         TabEntry te;
         te.I = kNoVote;
         te.g = 0.f;
-        if (!GENERAL_ONLY && rr < nrows && ((umask >> l) & 1u)) te = p.w.tab[l * ax.n_qpt + i0 + rr];
+        if (rr < nrows && ((umask >> l) & 1u)) te = p.w.tab[l * ax.n_qpt + i0 + rr];
         tab[q] = te;
     }
     for (int q = threadIdx.x; q < R; q += TPB) kq[q] = q < nrows ? p.w.kq32[i0 + q] : 0.f;
@@ -248,27 +237,23 @@ __global__ void __launch_bounds__(TPB) scatter_kernel(VoteParams p)
             int ja = 0, jb = -1;   // inclusive J window, possibly beyond [0, nphi)
             bool none = lend == lstart;
             if (!none && ((umask >> l) & 1u)) {
-                if (GENERAL_ONLY) {
-                    none = true;   // the gather kernel votes for this layer
+                // vote bin J - I - (f < g) lies in [J0, J0 + W) only for J in
+                // [J0 + min I, J0 + W + max I] over the slab's voting rows
+                int imin = INT_MAX, imax = INT_MIN;
+                for (int rr = 0; rr < nrows; ++rr) {
+                    const int I = tab[l * R + rr].I;
+                    if (I != kNoVote) {
+                        imin = min(imin, I);
+                        imax = max(imax, I);
+                    }
+                }
+                if (imin > imax) {
+                    none = true;
                 } else {
-                    // vote bin J - I - (f < g) lies in [J0, J0 + W) only for J in
-                    // [J0 + min I, J0 + W + max I] over the slab's voting rows
-                    int imin = INT_MAX, imax = INT_MIN;
-                    for (int rr = 0; rr < nrows; ++rr) {
-                        const int I = tab[l * R + rr].I;
-                        if (I != kNoVote) {
-                            imin = min(imin, I);
-                            imax = max(imax, I);
-                        }
-                    }
-                    if (imin > imax) {
-                        none = true;
-                    } else {
-                        ja = J0 + imin;
-                        jb = J0 + W + imax;
-                        // votes of this window fall in [imin - imax - 1, W + imax - imin] of the tile
-                        if (imax - imin + 1 <= kTileMargin) atomicOr(&s_fast, 1u << l);
-                    }
+                    ja = J0 + imin;
+                    jb = J0 + W + imax;
+                    // votes of this window fall in [imin - imax - 1, W + imax - imin] of the tile
+                    if (imax - imin + 1 <= kTileMargin) atomicOr(&s_fast, 1u << l);
                 }
             } else if (!none && ax.n_d0) {
                 ja = 0;   // per-vote layer on a grid with a d0 axis: every hit of the layer
@@ -402,7 +387,7 @@ __global__ void __launch_bounds__(TPB) scatter_kernel(VoteParams p)
             if (cb + HS * 32 < total) fetch_hit(cb + HS * 32 + lane, pos_n, off_n, hh_n);
             const int l = (int)((hh.jl >> 16) & 0x1Fu);
             const int J = (int)(hh.jl & 0xFFFFu);
-            const bool table_hit = !GENERAL_ONLY && l < 16 && ((umask >> l) & 1u);
+            const bool table_hit = l < 16 && ((umask >> l) & 1u);
             // a table layer whose votes fall within the margins, one mask a word: the byte offset
             // of its column in a row of the tile (the vote then subtracts the row's shift in bytes)
             const bool fast_hit = CELL != 0 && !wrap && table_hit && ((s_fast >> l) & 1u);
@@ -420,7 +405,7 @@ __global__ void __launch_bounds__(TPB) scatter_kernel(VoteParams p)
                 const int k1 = heads ? __ffs(heads) - 1 : nvalid;
                 const int lr = __shfl_sync(0xFFFFFFFFu, l, k0);
                 const uint32_t lbit = 1u << lr;
-                if (!GENERAL_ONLY && ((umask >> lr) & 1u)) {
+                if ((umask >> lr) & 1u) {
                     const TabEntry te = tab[lr * R + (rowok ? rr : 0)];
                     const bool valid = rowok && te.I != kNoVote;
                     const float g = te.g;
@@ -529,12 +514,10 @@ __global__ void __launch_bounds__(TPB) scatter_kernel(VoteParams p)
     }
     if (qn) flush_refines();
     if (refined) atomicAdd(&s_refined, refined);
-    if (GENERAL_ONLY) pdl_enter();   // the gathered accumulator is complete
     __syncthreads();
 
     // flush the tile: 8 cells of a row per thread, consecutive threads on consecutive rows (one
-    // bank each in the column-major tile), one 16-byte store (ORed into the gathered layers' bits,
-    // or added to their counts, when only the layers of several radii were voted here)
+    // bank each in the column-major tile), one 16-byte store
     uint16_t *M = p.w.M + (int64_t)e * ax.n_qpt * nphi;
     const int v8 = W >> 3;
     for (int q = threadIdx.x; q < nrows * v8; q += TPB) {
@@ -544,15 +527,6 @@ __global__ void __launch_bounds__(TPB) scatter_kernel(VoteParams p)
             uint32_t cnt[8];
 #pragma unroll
             for (int k = 0; k < 8; ++k) cnt[k] = tile[(c8 * 8 + k) * pitch + rr];
-            if (GENERAL_ONLY) {
-                const uint4 old = *dst;
-                const uint32_t ow[4] = {old.x, old.y, old.z, old.w};
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    cnt[2 * k] += ow[k] & 0xFFFFu;
-                    cnt[2 * k + 1] += ow[k] >> 16;
-                }
-            }
             auto pack = [](uint32_t lo, uint32_t hi) { return min(lo, 65535u) | (min(hi, 65535u) << 16); };
             *dst = make_uint4(pack(cnt[0], cnt[1]), pack(cnt[2], cnt[3]), pack(cnt[4], cnt[5]), pack(cnt[6], cnt[7]));
             continue;
@@ -567,16 +541,424 @@ __global__ void __launch_bounds__(TPB) scatter_kernel(VoteParams p)
             v = make_uint4(tile[(c8 * 4) * pitch + rr], tile[(c8 * 4 + 1) * pitch + rr], tile[(c8 * 4 + 2) * pitch + rr],
                            tile[(c8 * 4 + 3) * pitch + rr]);
         }
-        if (GENERAL_ONLY) {
-            const uint4 old = *dst;
-            v.x |= old.x;
-            v.y |= old.y;
-            v.z |= old.z;
-            v.w |= old.w;
-        }
         *dst = v;
     }
     if (threadIdx.x == 0 && s_refined) atomicAdd(&p.w.stats[e].refined_votes, s_refined);
+}
+
+// The vote of layers whose hits lie at several radii, after the gather: ORed into (added to) the gathered
+// accumulator.  A CTA takes tiles of kGenRows rows x kGenCols columns, a lane a row, the tile's hits 32
+// at a time a warp, each broadcast to all lanes.  The detectors that need this have their modules near
+// a common radius, so instead of an arcsine per vote the lane holds, for its row and the layer, the
+// cubic of T(r) = Nphi asin(c(r) k) / (2 pi) around the layer's middle radius r0 (T(r0) in FP64, split
+// into a whole number and a fraction): a vote is three multiply-adds and a floor.  A (layer, row) takes
+// the cubic when its error over the layer's radii stays below kCubicErr bins (the fourth derivative of
+// asin, (9 x + 6 x^3) / (1 - x^2)^(7/2), at the largest x, bounds the remainder) and T moves by at most
+// kCubicSpan bins; r - r0 is exact, so with the roundings of f and of the sums a vote is known to
+// kCubicEps bins, and only votes closer than that to a bin edge are redone in FP64, 32 of a warp's queue
+// at a time.  Rows with |x| above kNearLimit on which the cubic will not do take the arcsine from its end,
+// asin|x| = pi/2 - 2 asin(sqrt((1 - |x|) / 2)), with 1 - |x| and the square root in two-float arithmetic
+// and the series of asin to the eleventh power: known to the same window (deciding the votes of |x| > 0.99
+// in FP64 instead put 60,000 of them on the 16 tiles of the largest |q/pT|, 260 us).  What is left (radii
+// far apart) evaluates asinf per vote with the wider window refine_eps.  Measured on the 100k-hit event
+// with radii +-0.5 cm: 511 us with asinf per vote and a CTA of eight warps a tile.  With no such layer it returns at once: a grid of at most one CTA per
+// SM strides over the tiles, so that an empty launch costs the same for one event and for a batch.
+constexpr int kGenRows = 32, kGenCols = 256, kGenThreads = 1024;
+constexpr double kCubicErr = 2e-5, kCubicSpan = 32.0;
+constexpr float kCubicEps = 2e-4f, kNearLimit = 0.85f;
+
+struct GeneralParams {
+    Axes ax;
+    Workspace w;
+    int n_spans, tiles_per_event;
+    float s32, refine_eps;
+};
+
+// Per (layer, row) of a tile: the negated cubic's fraction and coefficients, and I with the row's kind in
+// its low two bits (0: the layer's hits cannot vote, 1: cubic, 2: asinf per vote, 3: the arcsine from its
+// end, the row's |x| / r as two floats in the first two coefficients).
+struct GeneralSmem {
+    uint32_t tile[kGenCols * kGenRows];
+    uint4 hits[kGenThreads];                           // per warp: f, r - r0, column of J in the tile, staged position
+    uint2 queue[kGenThreads / 32 * kRefineQueue];      // per warp: staged position, row | layer << 16
+    float4 co[HOUGH_MAX_LAYERS * kGenRows];
+    int I[HOUGH_MAX_LAYERS * kGenRows];
+    float kq[kGenRows];
+};
+
+template <bool COUNTS>
+__global__ void __launch_bounds__(kGenThreads) general_kernel(GeneralParams p)
+{
+    // Nothing the predecessor (the gather) writes is read until a tile is flushed: the layer records,
+    // bucket offsets and sorted hits come from kernels that finished before the gather could launch.  So
+    // the votes are cast first, and the wait comes before the first flush.
+    extern __shared__ __align__(16) unsigned char general_smem[];
+    GeneralSmem &S = *reinterpret_cast<GeneralSmem *>(general_smem);
+    __shared__ int s_start[kMaxRanges], s_off[kMaxRanges], s_pre[kMaxRanges + 1];
+    __shared__ unsigned s_wrap;
+    __shared__ unsigned long long s_refined;
+    const Axes &ax = p.ax;
+    const int L = ax.n_layers, nphi = ax.n_phi, nkeys = L * nphi;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    LayerInfo li{};
+    if (lane < L) li = p.w.info[lane];
+    const unsigned gmask = __ballot_sync(0xFFFFFFFFu, lane < L && li.present && !li.uniform);
+    if (!gmask) {
+        pdl_enter();
+        return;
+    }
+    bool waited = false;
+    uint4 *hitbuf = S.hits + 32 * warp;
+    uint2 *rq = S.queue + kRefineQueue * warp;
+    const unsigned rowaddr = smem_u32(S.tile + lane);
+    for (int tile = blockIdx.x; tile < p.w.n_events * p.tiles_per_event; tile += gridDim.x) {
+        const int e = tile / p.tiles_per_event, t = tile - e * p.tiles_per_event;
+        const int slab = t / p.n_spans, span = t - slab * p.n_spans;
+        const int i0 = slab * kGenRows, nrows = min(kGenRows, ax.n_qpt - i0);
+        const int J0 = span * kGenCols, W = min(kGenCols, nphi - J0);
+        const int64_t hstart = p.w.hit_start[e];
+        const HotHit *hot = p.w.hot + hstart;
+        const ColdHit *cold = p.w.cold + hstart;
+        const int32_t *offs = p.w.offs + (int64_t)e * (nkeys + 1);
+        if (threadIdx.x == 0) {
+            s_wrap = 0u;
+            s_refined = 0ull;
+        }
+        __syncthreads();
+        for (int q = threadIdx.x; q < kGenCols * kGenRows / 4; q += kGenThreads)
+            reinterpret_cast<uint4 *>(S.tile)[q] = make_uint4(0u, 0u, 0u, 0u);
+        if (threadIdx.x < kGenRows) S.kq[threadIdx.x] = threadIdx.x < nrows ? p.w.kq32[i0 + threadIdx.x] : 0.f;
+        for (int q = threadIdx.x; q < L * kGenRows; q += kGenThreads) {
+            const int l = q / kGenRows, rr = q - l * kGenRows;
+            float4 co = make_float4(0.f, 0.f, 0.f, 0.f);
+            int kind = 0, I = 0;
+            if (((gmask >> l) & 1u) && rr < nrows) {
+                kind = 2;
+                const float rmin = __uint_as_float(p.w.radii->rmin[l]), rmax = __uint_as_float(p.w.radii->rmax[l]);
+                const float r0 = 0.5f * (rmin + rmax);
+                if (!ax.n_d0) {
+                    const double k = qpt_centre(ax, i0 + rr), ck = sagitta_coef(ax, 1.0) * k;   // x = ck r
+                    const double xm = fabs(ck) * (double)rmax;
+                    if (fabs(ck) * (double)rmin > 1.0 + 1e-9) {
+                        kind = 0;
+                    } else if (xm <= 0.97 && rmin >= 0.5f * r0 && rmax <= 2.f * r0) {
+                        const double s = (double)ax.n_phi * kInvTwoPi, x = ck * (double)r0;
+                        const double y = 1.0 - x * x, rs = rsqrt(y), dx = ck * 0.5 * (double)(rmax - rmin) * 1.0001;
+                        const float ym = (float)(1.0 - xm * xm), xf = (float)xm;
+                        const float d4 = (9.f * xf + 6.f * xf * xf * xf) * rsqrtf(ym) / (ym * ym * ym);
+                        const float dx2 = (float)(dx * dx);
+                        const double d1 = s * ck * rs;
+                        if ((float)s * dx2 * dx2 * d4 * (1.01f / 24.f) <= (float)kCubicErr &&
+                            s * fabs(dx) * rsqrtf(ym) <= kCubicSpan) {
+                            const double T = s * asin(x), fI = floor(T);
+                            kind = 1;
+                            I = (int)fI;
+                            co.x = -(float)(T - fI);
+                            co.y = -(float)d1;
+                            co.z = -(float)(0.5 * s * ck * ck * x * rs * rs * rs);
+                            co.w = -(float)(s * ck * ck * ck * (1.0 + 2.0 * x * x) * rs * rs * rs * rs * rs * (1.0 / 6.0));
+                        }
+                    }
+                    if (kind == 2 && fabs(ck) * (double)rmin >= (double)kNearLimit) {
+                        kind = 3;
+                        I = k < 0.0 ? -1 : 1;
+                        co.x = (float)fabs(ck);
+                        co.y = (float)(fabs(ck) - (double)co.x);
+                    }
+                }
+            }
+            S.co[q] = co;
+            S.I[q] = I * 4 + kind;
+        }
+        // per layer, the hits that can vote into this tile: a cyclic window [ja, jb] of phi bins J, as one
+        // or two ranges of the sorted hits; s_off[q] takes the J of range q's hits to columns of the tile
+        if (threadIdx.x < HOUGH_MAX_LAYERS) {
+            const int l = threadIdx.x;
+            int nr = 0, st[2] = {0, 0}, ln[2] = {0, 0}, of[2] = {0, 0};
+            if ((gmask >> l) & 1u) {
+                const int lstart = offs[l * nphi], lend = offs[(l + 1) * nphi];
+                int ja = 0, jb = nphi;   // a grid with a d0 axis: every hit of the layer
+                if (!ax.n_d0) {
+                    // bound asin(c k) over the layer's radius range and the slab's rows
+                    const float c_lo = 0.15f * (float)ax.b / 100.f * __uint_as_float(p.w.radii->rmin[l]) * 0.999f;
+                    const float c_hi = 0.15f * (float)ax.b / 100.f * __uint_as_float(p.w.radii->rmax[l]) * 1.001f;
+                    const float k_a = p.w.kq32[i0], k_b = p.w.kq32[i0 + nrows - 1];
+                    const float xs[4] = {c_lo * k_a, c_lo * k_b, c_hi * k_a, c_hi * k_b};
+                    float amin = 2.f, amax = -2.f;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const float a = asinf(fminf(fmaxf(xs[u], -1.f), 1.f));
+                        amin = fminf(amin, a);
+                        amax = fmaxf(amax, a);
+                    }
+                    ja = (int)floorf(J0 + p.s32 * amin) - 2;
+                    jb = (int)floorf(J0 + W + p.s32 * amax) + 2;
+                }
+                if (lend > lstart && jb - ja + 1 >= nphi) {
+                    nr = 1;
+                    st[0] = lstart;
+                    ln[0] = lend - lstart;
+                    of[0] = -J0;
+                    atomicOr(&s_wrap, 1u << l);
+                } else if (lend > lstart) {
+                    const int a = ((ja % nphi) + nphi) % nphi, b = ((jb % nphi) + nphi) % nphi;
+                    of[0] = ja - a - J0;
+                    st[0] = offs[l * nphi + a];
+                    if (a <= b) {
+                        nr = 1;
+                        ln[0] = offs[l * nphi + b + 1] - st[0];
+                    } else {
+                        nr = 2;
+                        ln[0] = lend - st[0];
+                        st[1] = lstart;
+                        ln[1] = offs[l * nphi + b + 1] - lstart;
+                        of[1] = ja - a + nphi - J0;
+                    }
+                }
+            }
+            s_start[2 * l] = st[0];
+            s_start[2 * l + 1] = st[1];
+            s_off[2 * l] = of[0];
+            s_off[2 * l + 1] = of[1];
+            s_pre[2 * l] = nr >= 1 ? ln[0] : 0;   // lengths for now
+            s_pre[2 * l + 1] = nr >= 2 ? ln[1] : 0;
+        }
+        __syncthreads();
+        if (warp == 0) {   // (kMaxRanges is a warp's lanes)
+            const int len = s_pre[lane];
+            int incl = len;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int v = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+                if (lane >= d) incl += v;
+            }
+            s_pre[lane] = incl - len;
+            if (lane == 31) s_pre[kMaxRanges] = incl;
+        }
+        __syncthreads();
+        const int total = s_pre[kMaxRanges];
+        const unsigned wrapm = s_wrap;
+        const bool rowok = lane < nrows;
+        const int i = i0 + lane;
+        const float kqr = S.kq[lane];
+        unsigned refined = 0;
+        int qn = 0;   // the warp's queued votes (the same in every lane)
+        auto cast = [&](int jt, unsigned lbit) {
+            if (COUNTS) asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(rowaddr + (unsigned)jt * (4u * kGenRows)) : "memory");
+            else asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(rowaddr + (unsigned)jt * (4u * kGenRows)), "r"(lbit) : "memory");
+        };
+        auto flush_queue = [&]() {
+            __syncwarp();
+            for (int u = lane; u < qn; u += 32) {
+                const uint2 q = rq[u];
+                const int row = (int)(q.y & 0xFFFFu);
+                const ColdHit ch = cold[q.x];
+                const double x64 = __dmul_rn(sagitta_coef(ax, (double)ch.r), qpt_centre(ax, i0 + row));
+                const int jt = exact_bin(ax, (double)ch.phi, x64) - J0;
+                if ((unsigned)jt < (unsigned)W) {
+                    if (COUNTS) atomicAdd(&S.tile[jt * kGenRows + row], 1u);
+                    else atomicOr(&S.tile[jt * kGenRows + row], 1u << (q.y >> 16));
+                }
+            }
+            __syncwarp();
+            qn = 0;
+        };
+        // a vote too close to a bin edge waits in the queue
+        auto enqueue = [&](bool need, unsigned pos, int l) {
+            const unsigned rb = __ballot_sync(0xFFFFFFFFu, need);
+            if (need) rq[qn + __popc(rb & ((1u << lane) - 1u))] = make_uint2(pos, (uint32_t)lane | ((uint32_t)l << 16));
+            qn += __popc(rb);
+            refined += (unsigned)__popc(rb);
+            if (qn >= 32) flush_queue();   // at most 63 queued
+        };
+        for (int cb = warp * 32; cb < total; cb += kGenThreads) {
+            const int nvalid = min(32, total - cb);
+            int l = HOUGH_MAX_LAYERS, pos = 0;
+            HotHit hh{0.f, 0.f, 0u, 1u};
+            if (lane < nvalid) {
+                const int v = cb + lane;
+                int q = 0;   // the range holding v: the last q with s_pre[q] <= v
+#pragma unroll
+                for (int step = 16; step > 0; step >>= 1)
+                    if (s_pre[q + step] <= v) q += step;
+                pos = s_start[q] + (v - s_pre[q]);
+                hh = hot[pos];
+                const float r = cold[pos].r;
+                l = (int)((hh.jl >> 16) & 0xFu);
+                const float r0 = 0.5f * (__uint_as_float(p.w.radii->rmin[l]) + __uint_as_float(p.w.radii->rmax[l]));
+                hitbuf[lane] = make_uint4(__float_as_uint(hh.f), __float_as_uint(r - r0),
+                                          (uint32_t)((int)(hh.jl & 0xFFFFu) + s_off[q]), (uint32_t)pos);
+            }
+            __syncwarp();
+            // runs of hits of one layer (the ranges are in layer order)
+            const int lprev = __shfl_up_sync(0xFFFFFFFFu, l, 1);
+            unsigned heads = __ballot_sync(0xFFFFFFFFu, lane < nvalid && (lane == 0 || l != lprev));
+            while (heads) {
+                const int k0 = __ffs(heads) - 1;
+                heads &= heads - 1u;
+                const int k1 = heads ? __ffs(heads) - 1 : nvalid;
+                const int lr = __shfl_sync(0xFFFFFFFFu, l, k0);
+                const unsigned lbit = 1u << lr;
+                const bool wrap = (wrapm >> lr) & 1u;
+                const float4 co = S.co[lr * kGenRows + lane];
+                const int Ik = S.I[lr * kGenRows + lane];
+                const int kind = rowok ? Ik & 3 : 0, I = Ik >> 2;
+                if (__any_sync(0xFFFFFFFFu, kind == 1)) {
+                    // a lane of another kind has its votes fall far outside the tile
+                    const int shift = (kind == 1 ? -I : -(1 << 28)) - 0x4B400000;
+                    const float half_less = 0.5f - kCubicEps;
+                    // four hits at a time without a branch: a vote outside the tile or too close to an edge is
+                    // predicated off, and the four are looked at again when one of them was close
+                    auto four = [&](auto wrap_type, const int k, const int n) {
+                        constexpr bool wraps = decltype(wrap_type)::value;
+                        uint4 h[4];
+                        float dist[4];
+                        int jt[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) h[u] = hitbuf[k + min(u, n - 1)];
+                        float far = 0.f;
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const float x = __uint_as_float(h[u].y);
+                            const float v = fmaf(x, fmaf(x, fmaf(x, co.w, co.z), co.y), __uint_as_float(h[u].x)) + co.x;
+                            const float fl = __fadd_rd(v, 12582912.f);   // 1.5 * 2^23: the sum's low bits are floor(v)
+                            dist[u] = fabsf((v - (fl - 12582912.f)) - 0.5f);
+                            far = fmaxf(far, dist[u]);
+                            jt[u] = (int)h[u].z + __float_as_int(fl) + shift;
+                            if (wraps) {   // every hit of the layer: the column modulo Nphi
+                                jt[u] += jt[u] + J0 < 0 ? nphi : 0;
+                                jt[u] -= jt[u] + J0 >= nphi ? nphi : 0;
+                            }
+                            if (u >= n) jt[u] = -1;   // (n: the same for the whole warp)
+                            const unsigned addr = rowaddr + (unsigned)jt[u] * (4u * kGenRows);
+                            if (COUNTS)
+                                asm volatile("{\n\t.reg .pred p, q;\n\tsetp.gt.f32 q, %1, %2;\n\t"
+                                             "setp.lt.and.u32 p, %3, %4, !q;\n\t@p red.shared.add.u32 [%0], 1;\n\t}"
+                                             ::"r"(addr), "f"(dist[u]), "f"(half_less), "r"(jt[u]), "r"(W) : "memory");
+                            else
+                                asm volatile("{\n\t.reg .pred p, q;\n\tsetp.gt.f32 q, %1, %2;\n\t"
+                                             "setp.lt.and.u32 p, %3, %4, !q;\n\t@p red.shared.or.b32 [%0], %5;\n\t}"
+                                             ::"r"(addr), "f"(dist[u]), "f"(half_less), "r"(jt[u]), "r"(W), "r"(lbit) : "memory");
+                        }
+                        if (!__any_sync(0xFFFFFFFFu, far > half_less)) return;
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            enqueue(u < n && kind == 1 && dist[u] > half_less &&
+                                        (wraps || (unsigned)(jt[u] + 1) <= (unsigned)(W + 1)), h[u].w, lr);
+                    };
+                    if (wrap) {
+                        for (int k = k0; k < k1; k += 4) four(std::true_type{}, k, min(4, k1 - k));
+                    } else {
+                        int k = k0;
+                        for (; k + 4 <= k1; k += 4) four(std::false_type{}, k, 4);
+                        if (k < k1) four(std::false_type{}, k, k1 - k);
+                    }
+                }
+                if (__any_sync(0xFFFFFFFFu, kind == 3)) {
+                    const float r0 = 0.5f * (__uint_as_float(p.w.radii->rmin[lr]) + __uint_as_float(p.w.radii->rmax[lr]));
+                    const float s2h = 2.f * ax.u_hi, s2l = 2.f * ax.u_lo, sg = (float)I;
+                    for (int k = k0; k < k1; ++k) {
+                        const uint4 h = hitbuf[k];
+                        const uint32_t rows = __shfl_sync(0xFFFFFFFFu, hh.rows, k);
+                        const bool act = kind == 3 && i >= (int)(rows & 0xFFFFu) && i <= (int)(rows >> 16);
+                        const float r = r0 + __uint_as_float(h.y);   // exact: the difference was
+                        // |x| = xp.x + xp.y, then w = (1 - |x|) / 2 = wv.x + wv.y
+                        float2 xp = two_prod(r, co.x);
+                        xp.y = fmaf(r, co.y, xp.y);
+                        float2 wv = two_sum(1.f - xp.x, -xp.y);
+                        wv.x = fmaxf(0.5f * wv.x, 1e-30f);
+                        wv.y *= 0.5f;
+                        const float rs = rsqrtf(wv.x), tt = wv.x * rs;   // tt + tl = sqrt(w)
+                        const float tl = 0.5f * rs * (fmaf(-tt, tt, wv.x) + wv.y);
+                        float z = fmaf(wv.x, 945.f / 42240.f, 105.f / 3456.f);
+                        z = fmaf(wv.x, z, 15.f / 336.f);
+                        z = fmaf(wv.x, z, 3.f / 40.f);
+                        z = fmaf(wv.x, z, 1.f / 6.f);
+                        const float small = fmaf(tt * wv.x, z, tl);      // asin(sqrt(w)) = tt + small
+                        // Q = Nphi / (2 pi) 2 asin(sqrt(w)); T = +-(Nphi / 4 - Q)
+                        float2 Q = two_prod(tt, s2h);
+                        Q.y += fmaf(tt, s2l, small * s2h);
+                        const float fq = floorf(Q.x);
+                        const float v = fmaf(sg, (Q.x - fq) + Q.y, __uint_as_float(h.x));
+                        const float fl = floorf(v);
+                        const float d = v - fl;
+                        int jt = (int)h.z + I * ((int)fq - (nphi >> 2)) + (int)fl;
+                        if (wrap) {
+                            jt += jt + J0 < 0 ? nphi : 0;
+                            jt -= jt + J0 >= nphi ? nphi : 0;
+                        }
+                        const bool near = act && fabsf(d - 0.5f) > 0.5f - kCubicEps &&
+                                          (wrap || (unsigned)(jt + 1) <= (unsigned)(W + 1));
+                        if (act && !near && (unsigned)jt < (unsigned)W) cast(jt, lbit);
+                        if (__any_sync(0xFFFFFFFFu, near)) enqueue(near, h.w, lr);
+                    }
+                }
+                if (!__any_sync(0xFFFFFFFFu, kind == 2)) continue;
+                for (int k = k0; k < k1; ++k) {
+                    const uint4 h = hitbuf[k];
+                    const float c = __shfl_sync(0xFFFFFFFFu, hh.c, k);
+                    const uint32_t rows = __shfl_sync(0xFFFFFFFFu, hh.rows, k);
+                    bool act = kind == 2 && i >= (int)(rows & 0xFFFFu) && i <= (int)(rows >> 16);
+                    int jt = 0;
+                    if (ax.n_d0) {
+                        // a grid with a d0 axis: every vote in FP64, in the definition's order
+                        if (act) {
+                            const ColdHit ch = cold[h.w];
+                            int j;
+                            act = exact_vote(ax, (double)ch.r, (double)ch.phi, i, &j);
+                            jt = j - J0;
+                        }
+                    } else {
+                        const float x = fminf(fmaxf(c * kqr, -1.f), 1.f);
+                        const float vq = fmaf(-asinf(x), p.s32, __uint_as_float(h.x));
+                        const float fl = floorf(vq);
+                        const float d = vq - fl;
+                        jt = (int)h.z + (int)fl;
+                        if (wrap) {
+                            jt += jt + J0 < 0 ? nphi : 0;
+                            jt -= jt + J0 >= nphi ? nphi : 0;
+                        }
+                        const bool need = act && (d < p.refine_eps || d > 1.f - p.refine_eps || fabsf(x) > kRefineXLim);
+                        if (__any_sync(0xFFFFFFFFu, need)) enqueue(need, h.w, lr);
+                        act = act && !need;
+                    }
+                    if (act && (unsigned)jt < (unsigned)W) cast(jt, lbit);
+                }
+            }
+            __syncwarp();   // the buffer is read before the next chunk overwrites it
+        }
+        if (qn) flush_queue();
+        if (lane == 0 && refined) atomicAdd(&s_refined, (unsigned long long)refined);
+        if (!waited) pdl_enter();   // the gathered accumulator is complete
+        waited = true;
+        __syncthreads();
+        // flush the tile: 8 cells of a row per thread, consecutive threads on consecutive rows
+        uint16_t *M = p.w.M + (int64_t)e * ax.n_qpt * nphi;
+        if (total)
+            for (int q = threadIdx.x; q < (W >> 3) * kGenRows; q += kGenThreads) {
+                const int c8 = q / kGenRows, rr = q - c8 * kGenRows;
+                if (rr >= nrows) continue;
+                uint32_t m[8], any = 0u;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    m[k] = S.tile[(c8 * 8 + k) * kGenRows + rr];
+                    any |= m[k];
+                }
+                if (!any) continue;
+                uint4 *dst = reinterpret_cast<uint4 *>(M + (int64_t)(i0 + rr) * nphi + J0 + c8 * 8);
+                const uint4 old = *dst;
+                const uint32_t ow[4] = {old.x, old.y, old.z, old.w};
+                uint32_t v[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    v[k] = COUNTS ? min((ow[k] & 0xFFFFu) + m[2 * k], 65535u) | min((ow[k] >> 16) + m[2 * k + 1], 65535u) << 16
+                                  : ow[k] | m[2 * k] | m[2 * k + 1] << 16;
+                *dst = make_uint4(v[0], v[1], v[2], v[3]);
+            }
+        if (threadIdx.x == 0 && s_refined) atomicAdd(&p.w.stats[e].refined_votes, s_refined);
+        __syncthreads();   // the tile and the windows are free
+    }
+    if (!waited) pdl_enter();
 }
 
 // Gather: one tile of `rows` rows x `cols` columns of the accumulator from the per-bucket f
@@ -1479,23 +1861,23 @@ __global__ void copy_candidates_kernel(Workspace w, hough_candidate *out, long l
         dst[q] = src[q];
 }
 
-template <int TPB, bool GENERAL_ONLY, int CELL>
+template <int TPB, int CELL>
 cudaError_t launch_scatter(const VoteParams &p, size_t smem, int grid, cudaStream_t stream)
 {
-    cudaError_t err = cudaFuncSetAttribute(scatter_kernel<TPB, GENERAL_ONLY, CELL>,
+    cudaError_t err = cudaFuncSetAttribute(scatter_kernel<TPB, CELL>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err) return err;
-    return launch_chained(scatter_kernel<TPB, GENERAL_ONLY, CELL>, dim3(grid), dim3(TPB), smem, stream, p);
+    return launch_chained(scatter_kernel<TPB, CELL>, dim3(grid), dim3(TPB), smem, stream, p);
 }
 
-template <bool GENERAL_ONLY, int CELL>
+template <int CELL>
 cudaError_t launch_scatter_tpb(const VoteParams &p, int threads, size_t smem, int grid, cudaStream_t stream)
 {
     switch (threads) {
-    case 128: return launch_scatter<128, GENERAL_ONLY, CELL>(p, smem, grid, stream);
-    case 256: return launch_scatter<256, GENERAL_ONLY, CELL>(p, smem, grid, stream);
-    case 512: return launch_scatter<512, GENERAL_ONLY, CELL>(p, smem, grid, stream);
-    case 1024: return launch_scatter<1024, GENERAL_ONLY, CELL>(p, smem, grid, stream);
+    case 128: return launch_scatter<128, CELL>(p, smem, grid, stream);
+    case 256: return launch_scatter<256, CELL>(p, smem, grid, stream);
+    case 512: return launch_scatter<512, CELL>(p, smem, grid, stream);
+    case 1024: return launch_scatter<1024, CELL>(p, smem, grid, stream);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -1694,15 +2076,31 @@ cudaError_t launch_gather(const Axes &ax, const Workspace &w, const Tiling &t, c
     }
 }
 
+static cudaError_t launch_general(const Axes &ax, const Workspace &w, float refine_eps, cudaStream_t stream)
+{
+    GeneralParams p;
+    p.ax = ax;
+    p.w = w;
+    p.n_spans = (ax.n_phi + kGenCols - 1) / kGenCols;
+    p.tiles_per_event = ((ax.n_qpt + kGenRows - 1) / kGenRows) * p.n_spans;
+    p.s32 = (float)(ax.n_phi * kInvTwoPi);
+    p.refine_eps = refine_eps;
+    auto kernel = ax.counts ? general_kernel<true> : general_kernel<false>;
+    cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GeneralSmem));
+    if (err) return err;
+    const int grid = (int)std::min<int64_t>((int64_t)w.n_events * p.tiles_per_event, 152);
+    return launch_chained(kernel, dim3(grid), dim3(kGenThreads), sizeof(GeneralSmem), stream, p);
+}
+
 cudaError_t launch_scatter(const Axes &ax, const Workspace &w, const Tiling &t, float refine_eps, bool general_only,
                            cudaStream_t stream)
 {
+    if (general_only) return launch_general(ax, w, refine_eps, stream);
     const VoteParams p = vote_params(ax, w, t, refine_eps);
     const int grid = w.n_events * p.tiles_per_event;
     if (ax.counts) {
         const size_t smem = scatter_smem_bytes(ax, t, true);
-        return general_only ? launch_scatter_tpb<true, 2>(p, t.threads, smem, grid, stream)
-                            : launch_scatter_tpb<false, 2>(p, t.threads, smem, grid, stream);
+        return launch_scatter_tpb<2>(p, t.threads, smem, grid, stream);
     }
     // a mask a word when that tile fits (no shift to place the bit), else two a word
     static std::atomic<int> optin{0};
@@ -1715,11 +2113,9 @@ cudaError_t launch_scatter(const Axes &ax, const Workspace &w, const Tiling &t, 
     }
     const size_t wide = scatter_smem_bytes(ax, t, true);
     if (wide + 1024 <= (size_t)m)
-        return general_only ? launch_scatter_tpb<true, 1>(p, t.threads, wide, grid, stream)
-                            : launch_scatter_tpb<false, 1>(p, t.threads, wide, grid, stream);
+        return launch_scatter_tpb<1>(p, t.threads, wide, grid, stream);
     const size_t smem = scatter_smem_bytes(ax, t, false);
-    return general_only ? launch_scatter_tpb<true, 0>(p, t.threads, smem, grid, stream)
-                        : launch_scatter_tpb<false, 0>(p, t.threads, smem, grid, stream);
+    return launch_scatter_tpb<0>(p, t.threads, smem, grid, stream);
 }
 
 cudaError_t launch_vote(const Axes &ax, const Workspace &w, const Tiling &t, float refine_eps,
