@@ -88,9 +88,9 @@ typedef struct hough_geometry {
  * 1 <= threshold <= 16 (layer accumulator) or <= 65535 (count accumulator);
  * 1 <= n_cot, n_z0 <= 256 and n_cot * n_z0 <= 16384;
  * qpt_min < qpt_max, cot_min < cot_max, z0_min_cm < z0_max_cm.
- * With the count accumulator HOUGH_VOTE_GATHER counts per cell the hits of the
- * two buckets its votes come from, and HOUGH_VOTE_SCATTER is the shared-memory
- * atomic scatter; both give the same counts.
+ * The count accumulator is filled by the shared-memory atomic scatter, with the
+ * tile of the tiling under HOUGH_VOTE_SCATTER and one the library chooses under
+ * HOUGH_VOTE_GATHER; both give the same counts.
  *
  * Non-prompt tracks (n_d0 > 0): a third axis of n_d0 bins of the signed
  * transverse impact parameter d0 over [d0_min_cm, d0_max_cm).  A track whose
@@ -271,10 +271,9 @@ int hough_process(hough_ctx *ctx, const float *r, const float *phi, const float 
  * n_phi * 2 bytes of shared memory.
  * The peak search works on bands of band_rows rows.
  *
- * With the count accumulator the gather counts its tile of gather_rows x gather_cols cells in
- * 32-bit shared counters (gather_rows * gather_cols * 4 bytes plus a staging slot of at least
- * 16 KB must fit in shared memory) and the scatter's tile holds 32-bit counters; both saturate
- * to 16 bits when the tile is written out.
+ * With the count accumulator a tile holds 32-bit counters, saturated to 16 bits when it is
+ * written out (a gather tile must still be one that gather_rows * gather_cols * 4 bytes plus at
+ * least 16 KB of shared memory would hold).
  *
  * tile_phi must divide n_phi and be a multiple of 64; tile_qpt in 1..256; threads in
  * {128, 256, 512, 1024}; tile_qpt * tile_phi * 2 bytes (4 with the count accumulator) must fit

@@ -120,6 +120,7 @@ int hough_batch_create(const hough_geometry *geometry, const hough_binning *binn
     const int64_t E = limits->max_events, H = limits->max_hits, C = limits->max_candidates, Mm = limits->max_members;
     const int nkeys = n_keys(ax);
     Workspace &w = b->w;
+    w.table_chunks = 1;
     w.max_cand = (int)C;
     w.max_members = (int)Mm;
     w.n_hits_total = -1;           // read on the device
@@ -138,7 +139,7 @@ int hough_batch_create(const hough_geometry *geometry, const hough_binning *binn
         A(b->alloc(&w.gsort, (size_t)ax.n_layers * ax.n_qpt)); A(b->alloc(&w.rankt, (size_t)ax.n_layers * ax.n_qpt));
     }
     A(b->alloc(&w.radii, 1)); A(b->alloc(&w.info, HOUGH_MAX_LAYERS)); A(b->alloc(&w.memo, 1));
-    A(b->alloc(&w.tab, (size_t)ax.n_layers * ax.n_qpt)); A(b->alloc(&w.arc, (size_t)ax.n_layers * ax.n_qpt));
+    A(b->alloc(&w.tab, (size_t)ax.n_layers * ax.n_qpt));
     A(b->alloc(&w.zco, (size_t)ax.n_layers * ax.n_qpt));
     A(b->alloc(&w.kq32, ax.n_qpt));
     A(b->alloc(&w.M, (size_t)E * ax.n_qpt * ax.n_phi));
@@ -271,7 +272,7 @@ int hough::batch_run(hough_batch *b, const float *r, const float *phi, const flo
         it = b->graphs.emplace(n_events, exec).first;
     }
     BCU(cudaGraphLaunch(it->second, s), "graph launch failed");
-    note_launches(kStageLaunches + kVoteLaunches + kPeakLaunches + kStage2Launches);
+    note_launches(kStageLaunches + vote_launches(b->ax, b->tiling.vote_mode) + kPeakLaunches + kStage2Launches);
     b->n_events = n_events;
     b->ran = true;
     return HOUGH_OK;
@@ -349,7 +350,7 @@ int hough_batch_profile(hough_batch *b, const float *r, const float *phi, const 
     if (!e) e = cudaEventRecord(ev[6], s);
     if (!e) e = cudaStreamSynchronize(s);
     if (e) return done(bfail(HOUGH_ECUDA, "profiled batch run failed"));
-    note_launches(kStageLaunches + kVoteLaunches + kPeakLaunches + kStage2Launches);
+    note_launches(kStageLaunches + vote_launches(b->ax, b->tiling.vote_mode) + kPeakLaunches + kStage2Launches);
     b->n_events = n_events;
     b->ran = true;
     float ms[6];

@@ -244,9 +244,10 @@ int check_tiling_impl(const Axes &ax, int device, const hough_tiling *t)
         return fail(HOUGH_EINVAL, "band of %d rows needs %zu bytes of shared memory, the device allows %d",
                     t->band_rows, band_smem_bytes(ax, t->band_rows), max_smem);
     if (ax.counts && t->vote_mode == HOUGH_VOTE_GATHER) {
-        if (gather_count_smem_bytes(ax, tt) + 1024 > (size_t)max_smem)
-            return fail(HOUGH_EINVAL, "count gather tile needs %zu bytes of shared memory, the device allows %d",
-                        gather_count_smem_bytes(ax, tt), max_smem);
+        // (the documented size of a count tile; the vote itself chooses a tile of its own)
+        const size_t base = (size_t)ax.n_layers * (tt.gather_cols + 131) * 4, bytes = std::max(base + 16384, (size_t)96 * 1024);
+        if (bytes + 1024 > (size_t)max_smem)
+            return fail(HOUGH_EINVAL, "count gather tile needs %zu bytes of shared memory, the device allows %d", bytes, max_smem);
     }
     if (gather_smem_bytes(ax, tt) + 1024 > (size_t)max_smem)
         return fail(HOUGH_EINVAL, "gather tile needs %zu bytes of shared memory, the device allows %d",
@@ -394,7 +395,7 @@ int enqueue_vote(hough_ctx *c, const float *r, const float *phi, const float *z,
     if (c->timing) { CU(cudaEventRecord(c->ev[2], s), "event"); c->timed |= 4; }
     CU(launch_scatter(c->ax, c->w, c->tiling, c->refine_eps, c->tiling.vote_mode != HOUGH_VOTE_SCATTER, s), "vote kernel");
     if (c->timing) { CU(cudaEventRecord(c->ev[3], s), "event"); c->timed |= 8; }
-    g_launches += kStageLaunches - (clear ? 0 : 1) + (c->tiling.vote_mode == HOUGH_VOTE_SCATTER ? 1 : kVoteLaunches);
+    g_launches += kStageLaunches - (clear ? 0 : 1) + vote_launches(c->ax, c->tiling.vote_mode);
     c->stage = 1;
     return HOUGH_OK;
 }
@@ -498,6 +499,7 @@ int hough_create(const hough_geometry *geometry, const hough_binning *binning, c
     const int nkeys = n_keys(ax);
     Workspace &w = c->w;
     w.n_events = 1;
+    w.table_chunks = 1;
     w.max_cand = limits->max_candidates;
     w.max_members = limits->max_members;
     cudaError_t e = cudaSuccess;
@@ -513,7 +515,7 @@ int hough_create(const hough_geometry *geometry, const hough_binning *binning, c
     A(c->alloc(&w.hot, n)); A(c->alloc(&w.cold, n)); A(c->alloc(&w.fsort, n)); A(c->alloc(&w.zsort, n));
     A(c->alloc(&c->radii_buf[0], 1)); A(c->alloc(&c->radii_buf[1], 1));
     A(c->alloc(&w.info, HOUGH_MAX_LAYERS)); A(c->alloc(&w.memo, 1));
-    A(c->alloc(&w.tab, (size_t)ax.n_layers * ax.n_qpt)); A(c->alloc(&w.arc, (size_t)ax.n_layers * ax.n_qpt));
+    A(c->alloc(&w.tab, (size_t)ax.n_layers * ax.n_qpt));
     A(c->alloc(&w.zco, (size_t)ax.n_layers * ax.n_qpt));
     A(c->alloc(&w.kq32, ax.n_qpt));
     A(c->alloc(&w.M, (size_t)ax.n_qpt * ax.n_phi));

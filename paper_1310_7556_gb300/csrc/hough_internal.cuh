@@ -14,7 +14,7 @@
 //                             layer's table fractions g, as halves (gather vote of layer masks; kRankRows)
 //   hot[n], cold[n] (16 B)    staged hits sorted by (layer, J); cold holds r, phi, z, input index
 //   tab[L*Nq] (8 B)           per (layer, q/pT row): Nphi asin(x) / (2 pi) = I + g, for layers whose
-//                             hits share one radius; arc[L*Nq] the arc length s (FP64)
+//                             hits share one radius
 //   M[Nq*Nphi] (uint16)       stage-1 accumulator, row-major layer masks
 //   band_cands[n_bands*band_cap] (8 B)  peak candidates of each row band: row << 16 | column, mask
 //   cand_list (16 B)          the candidates of all events in order: row << 16 | column, mask, event,
@@ -161,9 +161,9 @@ struct Workspace {
     ColdHit *cold;
     LayerRadii *radii;            // batch-wide
     LayerInfo *info;              // HOUGH_MAX_LAYERS
-    TableMemo *memo;
+    TableMemo *memo;              // (null: the table is computed for every event, by table_chunks CTAs a layer)
+    int table_chunks;
     TabEntry *tab;                // n_layers * n_qpt
-    double *arc;                  // n_layers * n_qpt
     float4 *zco;                  // n_layers * n_qpt stage-2 terms {S hi, S lo, B hi, B lo} (may be null)
     float *kq32;                  // n_qpt: FP32 q/pT bin centres
     uint16_t *M;                  // n_events * n_qpt * n_phi
@@ -257,6 +257,7 @@ cudaError_t launch_member_index(const Workspace &w, int32_t *idx_out, int64_t to
 cudaError_t run_smem_or_bench(int device, int pattern, double ms, double *atomics_per_s, uint64_t *launches);
 
 size_t vote_smem_bytes(const Axes &ax, const Tiling &t);
+Tiling scatter_tiling(const Axes &ax, int n_events, Tiling t);   // t with the shared-atomic vote's tile chosen
 // Shared memory of the peak search over bands of band_rows rows.
 __host__ __device__ inline size_t band_smem_bytes(const Axes &ax, int band_rows)
 {
@@ -282,8 +283,6 @@ void public_tiling(const Tiling &t, hough_tiling *out);
 size_t gather_smem_bytes(const Axes &ax, const Tiling &t);
 // Dynamic shared memory of the fused vote and peak kernel: the band's masks and its two halo rows.
 size_t fused_smem_bytes(const Axes &ax, int band_rows);
-// Shared memory of the count accumulator's gather kernel.
-size_t gather_count_smem_bytes(const Axes &ax, const Tiling &t);
 size_t band_list_entries(const Axes &ax);
 int check_host_hits_for(const Axes &ax, const float *r, const float *phi, const float *z, const uint8_t *layer,
                         int64_t n);
@@ -308,7 +307,7 @@ void note_launches(uint64_t n);
 
 // Kernels launched by each enqueue function (for hough_kernel_launches).
 constexpr int kStageLaunches = 4;
-constexpr int kVoteLaunches = 2;
+inline int vote_launches(const Axes &ax, int vote_mode) { return vote_mode == HOUGH_VOTE_SCATTER || ax.counts ? 1 : 2; }
 // peak search, and the compaction's scan of the band counts and copy of the band lists
 constexpr int kCompactLaunches = 2;
 constexpr int kPeakLaunches = 1 + kCompactLaunches;

@@ -164,7 +164,8 @@ __global__ void __launch_bounds__(kStageThreads) stage_count_kernel(Axes ax, Wor
     count_epilogue(w, s_rmin, s_rmax);
 }
 
-// One CTA per layer: whether all the layer's hits share one radius, that radius's voting rows and
+// One CTA per layer (or `chunks` of them, each taking every chunks-th row, where no table is
+// kept between events and so none of them waits for the others' memo): whether all the layer's hits share one radius, that radius's voting rows and
 // whether the memoised table rows must be recomputed; then, for a uniform layer whose radius
 // changed, per row: T = Nphi asin(y) / (2 pi) split into I + g, y = sin(phi - phi0) of the row's
 // track (y = x for prompt tracks, the d0 relation on a grid with a d0 axis), the arc length from
@@ -224,7 +225,8 @@ __device__ void layer_ranks(const Axes &ax, const Workspace &w, const int l, con
     }
 }
 
-__device__ __forceinline__ void layer_table(const Axes &ax, const Workspace &w, const int l, int *s_tile)
+__device__ __forceinline__ void layer_table(const Axes &ax, const Workspace &w, const int l, const int chunk,
+                                            const int chunks, int *s_tile)
 {
     __shared__ LayerInfo s_li;
     __shared__ int s_dirty;
@@ -232,8 +234,12 @@ __device__ __forceinline__ void layer_table(const Axes &ax, const Workspace &w, 
         LayerInfo li;
         // every load of the decision at once (one round trip, not a chain of them)
         const unsigned rmin = w.radii->rmin[l], rmax = w.radii->rmax[l];
-        const int m_valid = w.memo->valid[l], m_lo = w.memo->lo[l], m_hi = w.memo->hi[l], m_nvote = w.memo->nvote[l];
-        const unsigned m_r = w.memo->r_bits[l];
+        int m_valid = 0, m_lo = 0, m_hi = 0, m_nvote = 0;
+        unsigned m_r = 0u;
+        if (w.memo) {
+            m_valid = w.memo->valid[l], m_lo = w.memo->lo[l], m_hi = w.memo->hi[l], m_nvote = w.memo->nvote[l];
+            m_r = w.memo->r_bits[l];
+        }
         li.present = (l < ax.n_layers) && rmax != 0u;
         li.uniform = !li.present || rmin == rmax;   // a layer without hits is trivially uniform
         li.lo = 1;
@@ -250,18 +256,21 @@ __device__ __forceinline__ void layer_table(const Axes &ax, const Workspace &w, 
                 } else {
                     row_range(ax, sagitta_coef(ax, (double)__uint_as_float(rmin)), &li.lo, &li.hi);
                 }
-                w.memo->r_bits[l] = rmin;
-                w.memo->lo[l] = li.lo;
-                w.memo->hi[l] = li.hi;
-                w.memo->valid[l] = 1;
+                if (chunks > 1) li.nvote = max(0, li.hi - li.lo + 1);   // prompt tracks: every row of the range votes
+                if (w.memo) {
+                    w.memo->r_bits[l] = rmin;
+                    w.memo->lo[l] = li.lo;
+                    w.memo->hi[l] = li.hi;
+                    w.memo->valid[l] = 1;
+                }
             } else {
                 li.lo = m_lo;   // the same radius as before: its rows are memoised
                 li.hi = m_hi;
                 li.nvote = m_nvote;
             }
         }
-        w.info[l] = li;
-        w.memo->dirty[l] = dirty;
+        if (chunk == 0) w.info[l] = li;
+        if (w.memo) w.memo->dirty[l] = dirty;
         s_li = li;
         s_dirty = dirty;
     }
@@ -274,7 +283,7 @@ __device__ __forceinline__ void layer_table(const Axes &ax, const Workspace &w, 
     const double r = (double)__uint_as_float(li.r_bits);
     const double t0 = __dadd_rn(ax.cot_min, __dmul_rn(0.5, ax.dt));
     int nvote = 0;
-    for (int i = threadIdx.x; i < ax.n_qpt; i += blockDim.x) {
+    for (int i = chunk + chunks * threadIdx.x; i < ax.n_qpt; i += chunks * blockDim.x) {
         const int q = l * ax.n_qpt + i;
         TabEntry te;
         te.I = kNoVote;
@@ -293,12 +302,11 @@ __device__ __forceinline__ void layer_table(const Axes &ax, const Workspace &w, 
                     te.I += 1;
                     te.g = 0.f;
                 }
-                s = track_arc(r, x, d0, y);
+                if (w.zco) s = track_arc(r, x, d0, y);
                 ++nvote;
             }
         }
         w.tab[q] = te;
-        w.arc[q] = s;
         if (w.zco) {
             // stage-2 terms of the layer's members on this row: the z0 coordinate of cot row m is
             // zscale (z - z0_min) - S - m B with S = zscale s t_0 and B = zscale s dt
@@ -308,11 +316,12 @@ __device__ __forceinline__ void layer_table(const Axes &ax, const Workspace &w, 
             w.zco[q] = make_float4(sh, (float)(S - (double)sh), bh, (float)(B - (double)bh));
         }
     }
+    if (chunks > 1) return;
     if (nvote) atomicAdd(&s_nvote, nvote);
     __syncthreads();
     if (threadIdx.x == 0) {
         w.info[l].nvote = s_nvote;
-        w.memo->nvote[l] = s_nvote;
+        if (w.memo) w.memo->nvote[l] = s_nvote;
     }
     // (kept with the table, whichever form of the vote this event takes)
     if (w.rankt) layer_ranks(ax, w, l, s_nvote, reinterpret_cast<float *>(s_tile));
@@ -448,7 +457,7 @@ __global__ void __launch_bounds__(kScanThreads) table_scan_kernel(Axes ax, Works
     const int scans = by_layer ? w.n_events * ax.n_layers : w.n_events;
     const int b = blockIdx.x;
     __shared__ int s_tile[kTileWords];
-    if (b >= scans) layer_table(ax, w, b - scans, s_tile);
+    if (b >= scans) layer_table(ax, w, (b - scans) / w.table_chunks, (b - scans) % w.table_chunks, w.table_chunks, s_tile);
     else if (by_layer) scan_layer(ax, w, b / ax.n_layers, b % ax.n_layers, s_tile);
     else scan_keys(ax, w, b, s_tile);
 }
@@ -661,7 +670,7 @@ cudaError_t launch_stage(const Axes &ax, const Workspace &w, cudaStream_t stream
     // a few events leave most SMs idle under one scan block each: then a block per (event, layer)
     const int by_layer = w.n_events <= 16 ? 1 : 0;
     const int scans = by_layer ? w.n_events * ax.n_layers : w.n_events;
-    if ((err = launch_chained(table_scan_kernel, dim3(scans + HOUGH_MAX_LAYERS), dim3(kScanThreads), 0, stream, ax, w,
+    if ((err = launch_chained(table_scan_kernel, dim3(scans + HOUGH_MAX_LAYERS * w.table_chunks), dim3(kScanThreads), 0, stream, ax, w,
                               by_layer)))
         return err;
     if ((err = mark(2))) return err;   // table_ms covers both; scan_ms stays empty

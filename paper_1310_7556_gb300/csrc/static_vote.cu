@@ -33,11 +33,9 @@ constexpr size_t kOffHitStart = 0;
 constexpr size_t kOffStats = align256(kOffHitStart + 2 * sizeof(int64_t));
 constexpr size_t kOffRadii = align256(kOffStats + sizeof(DevStats));
 constexpr size_t kOffInfo = align256(kOffRadii + sizeof(LayerRadii));
-constexpr size_t kOffMemo = align256(kOffInfo + HOUGH_MAX_LAYERS * sizeof(LayerInfo));
-constexpr size_t kOffKq = align256(kOffMemo + sizeof(TableMemo));
+constexpr size_t kOffKq = align256(kOffInfo + HOUGH_MAX_LAYERS * sizeof(LayerInfo));
 constexpr size_t kOffTab = align256(kOffKq + kStaticMaxQpt * sizeof(float));
-constexpr size_t kOffArc = align256(kOffTab + (size_t)HOUGH_MAX_LAYERS * kStaticMaxQpt * sizeof(TabEntry));
-constexpr size_t kOffCounts = align256(kOffArc + (size_t)HOUGH_MAX_LAYERS * kStaticMaxQpt * sizeof(double));
+constexpr size_t kOffCounts = align256(kOffTab + (size_t)HOUGH_MAX_LAYERS * kStaticMaxQpt * sizeof(TabEntry));
 constexpr size_t kOffOffs = align256(kOffCounts + (size_t)kStaticMaxKeys * sizeof(int32_t));
 constexpr size_t kOffKey = align256(kOffOffs + (size_t)(kStaticMaxKeys + 1) * sizeof(int32_t));
 constexpr size_t kOffRank = align256(kOffKey + (size_t)kStaticMaxHits * sizeof(int32_t));
@@ -125,10 +123,11 @@ extern "C" int hough_vote_static(const hough_geometry *g, const hough_binning *b
     w.stats = reinterpret_cast<DevStats *>(base + kOffStats);
     w.radii = reinterpret_cast<LayerRadii *>(base + kOffRadii);
     w.info = reinterpret_cast<LayerInfo *>(base + kOffInfo);
-    w.memo = reinterpret_cast<TableMemo *>(base + kOffMemo);
+    // no table is kept between calls, which may have other axes: each is computed by several CTAs a layer
+    // (one took 17 us of a 1,024-row call's 120), with the FP64 arcsine alone, as no stage 2 follows
+    w.table_chunks = ax.n_d0 ? 1 : 8;
     w.kq32 = reinterpret_cast<float *>(base + kOffKq);
     w.tab = reinterpret_cast<TabEntry *>(base + kOffTab);
-    w.arc = reinterpret_cast<double *>(base + kOffArc);
     w.counts = reinterpret_cast<int32_t *>(base + kOffCounts);
     w.offs = reinterpret_cast<int32_t *>(base + kOffOffs);
     w.key = reinterpret_cast<int32_t *>(base + kOffKey);
@@ -138,28 +137,19 @@ extern "C" int hough_vote_static(const hough_geometry *g, const hough_binning *b
     w.cold = reinterpret_cast<ColdHit *>(base + kOffCold);
     w.M = accumulator;
 
-    Tiling t;
-    t.tile_phi = b->n_phi < 256 ? b->n_phi : 256;
-    while (b->n_phi % t.tile_phi) t.tile_phi -= 64;
-    t.tile_qpt = b->n_qpt < 32 ? b->n_qpt : 32;
-    t.threads = 256;
+    Tiling t{};
     t.vote_mode = HOUGH_VOTE_SCATTER;   // the shared-atomic vote kernel alone: no bucket profile needed
-    t.band_rows = 4;
-    t.gather_rows = 4;
-    t.gather_cols = t.tile_phi;
-    t.gather_threads = 512;
+    t = scatter_tiling(ax, 1, t);
 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     // The array keeps the previous call's contents: reset what the kernels expect to start at zero.
-    // The arcsine-table memo is cleared too, since the previous call may have used other axes.
-    if (cudaMemsetAsync(base + kOffHitStart, 0, 2 * sizeof(int64_t), s) != cudaSuccess ||
-        cudaMemsetAsync(base + kOffMemo, 0, sizeof(TableMemo), s) != cudaSuccess)
+    if (cudaMemsetAsync(base + kOffHitStart, 0, 2 * sizeof(int64_t), s) != cudaSuccess)
         return fail(HOUGH_ECUDA, "clearing the fixed scratch failed");
     static_kq_kernel<<<(ax.n_qpt + 127) / 128, 128, 0, s>>>(ax, w.kq32);
     if (cudaGetLastError() != cudaSuccess) return fail(HOUGH_ECUDA, "q/pT centre kernel failed to launch");
     if (launch_stage(ax, w, s) != cudaSuccess) return fail(HOUGH_ECUDA, "staging kernels failed to launch");
     if (launch_vote(ax, w, t, refine_eps_for(ax), s) != cudaSuccess) return fail(HOUGH_ECUDA, "vote kernel failed to launch");
-    note_launches(1 + kStageLaunches + kVoteLaunches);
+    note_launches(1 + kStageLaunches + vote_launches(ax, t.vote_mode));
     if (device_error &&
         cudaMemcpyAsync(device_error, &w.stats->device_error, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s) != cudaSuccess)
         return fail(HOUGH_ECUDA, "copying the device error word failed");

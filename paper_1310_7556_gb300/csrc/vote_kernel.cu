@@ -1,7 +1,7 @@
 // Stage-1 vote (Sec. 4, first step; the A[B[i]] += 1 scatter of Sec. 8), accumulator flush and
 // the peak search over row bands (Sec. 4, second step).
 //
-// Three ways to fill the accumulator, selected per layer on the device:
+// Two ways to fill the accumulator, the second in two forms:
 //
 // 1. Gather (layers whose hits share one radius; every configured workload).  On row i every
 //    hit of such a layer votes at J - I_i - (f < g_i): its own bin coordinate J + f shifted by the
@@ -22,14 +22,9 @@
 //    adds its length with one atomicAdd from its first lane, and the flush saturates every counter
 //    to 16 bits -- the literal A[B[i]] += 1 of Sec. 8.  Table layers vote at
 //    J - I - (f < g); other layers take FP32 asinf per vote, and a vote within `refine_eps` of an
-//    edge (or with |x| > kRefineXLim) is recomputed in FP64 in the definition's order.  In the
-//    default (gather) mode this kernel handles only the layers whose radii differ and ORs its tile
-//    into the accumulator (adds it, with counts); in scatter mode it handles every layer and stores
-//    its tile.
-//
-// 3. Count gather (the count accumulator's gather mode): per cell and layer of one radius, the hits
-//    of bucket J' with f >= g_i and of bucket J' + 1 with f < g_i, counted from the sorted f values
-//    of the tile's window of buckets (gather_count_kernel).
+//    edge (or with |x| > kRefineXLim) is recomputed in FP64 in the definition's order.  It handles
+//    every layer and stores its tile: the vote in scatter mode and of counts in either mode.  After
+//    the gather of layer masks general_kernel adds the layers whose radii differ.
 //
 // Peaks: candidates of each band of band_rows rows (one row by default) go to a band list in
 // raster order; a scan of the band counts and a copy then concatenate the band lists of all events
@@ -546,8 +541,8 @@ __global__ void __launch_bounds__(TPB) scatter_kernel(VoteParams p)
     if (threadIdx.x == 0 && s_refined) atomicAdd(&p.w.stats[e].refined_votes, s_refined);
 }
 
-// The vote of layers whose hits lie at several radii, after the gather: ORed into (added to) the gathered
-// accumulator.  A CTA takes tiles of kGenRows rows x kGenCols columns, a lane a row, the tile's hits 32
+// The vote of layers whose hits lie at several radii, after the gather of layer masks: ORed into the
+// gathered accumulator.  A CTA takes tiles of kGenRows rows x kGenCols columns, a lane a row, the tile's hits 32
 // at a time a warp, each broadcast to all lanes.  The detectors that need this have their modules near
 // a common radius, so instead of an arcsine per vote the lane holds, for its row and the layer, the
 // cubic of T(r) = Nphi asin(c(r) k) / (2 pi) around the layer's middle radius r0 (T(r0) in FP64, split
@@ -586,7 +581,6 @@ struct GeneralSmem {
     float kq[kGenRows];
 };
 
-template <bool COUNTS>
 __global__ void __launch_bounds__(kGenThreads) general_kernel(GeneralParams p)
 {
     // Nothing the predecessor (the gather) writes is read until a tile is flushed: the layer records,
@@ -744,8 +738,7 @@ __global__ void __launch_bounds__(kGenThreads) general_kernel(GeneralParams p)
         unsigned refined = 0;
         int qn = 0;   // the warp's queued votes (the same in every lane)
         auto cast = [&](int jt, unsigned lbit) {
-            if (COUNTS) asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(rowaddr + (unsigned)jt * (4u * kGenRows)) : "memory");
-            else asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(rowaddr + (unsigned)jt * (4u * kGenRows)), "r"(lbit) : "memory");
+            asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(rowaddr + (unsigned)jt * (4u * kGenRows)), "r"(lbit) : "memory");
         };
         auto flush_queue = [&]() {
             __syncwarp();
@@ -755,10 +748,7 @@ __global__ void __launch_bounds__(kGenThreads) general_kernel(GeneralParams p)
                 const ColdHit ch = cold[q.x];
                 const double x64 = __dmul_rn(sagitta_coef(ax, (double)ch.r), qpt_centre(ax, i0 + row));
                 const int jt = exact_bin(ax, (double)ch.phi, x64) - J0;
-                if ((unsigned)jt < (unsigned)W) {
-                    if (COUNTS) atomicAdd(&S.tile[jt * kGenRows + row], 1u);
-                    else atomicOr(&S.tile[jt * kGenRows + row], 1u << (q.y >> 16));
-                }
+                if ((unsigned)jt < (unsigned)W) atomicOr(&S.tile[jt * kGenRows + row], 1u << (q.y >> 16));
             }
             __syncwarp();
             qn = 0;
@@ -831,14 +821,9 @@ __global__ void __launch_bounds__(kGenThreads) general_kernel(GeneralParams p)
                             }
                             if (u >= n) jt[u] = -1;   // (n: the same for the whole warp)
                             const unsigned addr = rowaddr + (unsigned)jt[u] * (4u * kGenRows);
-                            if (COUNTS)
-                                asm volatile("{\n\t.reg .pred p, q;\n\tsetp.gt.f32 q, %1, %2;\n\t"
-                                             "setp.lt.and.u32 p, %3, %4, !q;\n\t@p red.shared.add.u32 [%0], 1;\n\t}"
-                                             ::"r"(addr), "f"(dist[u]), "f"(half_less), "r"(jt[u]), "r"(W) : "memory");
-                            else
-                                asm volatile("{\n\t.reg .pred p, q;\n\tsetp.gt.f32 q, %1, %2;\n\t"
-                                             "setp.lt.and.u32 p, %3, %4, !q;\n\t@p red.shared.or.b32 [%0], %5;\n\t}"
-                                             ::"r"(addr), "f"(dist[u]), "f"(half_less), "r"(jt[u]), "r"(W), "r"(lbit) : "memory");
+                            asm volatile("{\n\t.reg .pred p, q;\n\tsetp.gt.f32 q, %1, %2;\n\t"
+                                         "setp.lt.and.u32 p, %3, %4, !q;\n\t@p red.shared.or.b32 [%0], %5;\n\t}"
+                                         ::"r"(addr), "f"(dist[u]), "f"(half_less), "r"(jt[u]), "r"(W), "r"(lbit) : "memory");
                         }
                         if (!__any_sync(0xFFFFFFFFu, far > half_less)) return;
 #pragma unroll
@@ -951,8 +936,7 @@ __global__ void __launch_bounds__(kGenThreads) general_kernel(GeneralParams p)
                 uint32_t v[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
-                    v[k] = COUNTS ? min((ow[k] & 0xFFFFu) + m[2 * k], 65535u) | min((ow[k] >> 16) + m[2 * k + 1], 65535u) << 16
-                                  : ow[k] | m[2 * k] | m[2 * k + 1] << 16;
+                    v[k] = ow[k] | m[2 * k] | m[2 * k + 1] << 16;
                 *dst = make_uint4(v[0], v[1], v[2], v[3]);
             }
         if (threadIdx.x == 0 && s_refined) atomicAdd(&p.w.stats[e].refined_votes, s_refined);
@@ -1471,161 +1455,6 @@ __global__ void __launch_bounds__(TPB) fused_kernel(GatherParams p)
     if (threadIdx.x == 0) w.band_counts[(int64_t)e * nb + band] = cnt;
 }
 
-// Count accumulator by gather.  On row i a layer of one radius adds to cell j the hits of bucket
-// J' = (j + I_i) mod Nphi with f >= g_i and the hits of bucket J' + 1 with f < g_i: exactly the
-// hits whose vote J - I_i - (f < g_i) is j, by the same FP32 comparison, so the same counts as the
-// scatter -- with no atomics.  A CTA owns `rows` x `cols` cells.  It first stages, for every layer
-// at once, the window of buckets its tile reads: the buckets' offsets (the bucket offsets are a
-// prefix sum already, so a window's are a difference of two, or three when it wraps around phi)
-// and the f values of their hits (the sorted hits of consecutive buckets are contiguous: one
-// range, or two when the window wraps).  Then a lane per cell sums, over the layers, the hits of
-// the two buckets its cell reads, and writes the saturated count.  A window too wide or too full
-// for its slot is read from global memory.  Layers whose hits lie at several radii are added by
-// the scatter kernel afterwards.
-constexpr int kCountWinPad = 128;    // window buckets beyond cols + 2 held in a layer's slot
-constexpr int kCountSmemBudget = 96 * 1024;
-
-__host__ __device__ inline int count_win_cap(int cols) { return cols + 2 + kCountWinPad; }
-
-template <int TPB>
-__global__ void __launch_bounds__(TPB) gather_count_kernel(GatherParams p, int fcap)
-{
-    pdl_enter();
-    extern __shared__ __align__(16) unsigned char count_smem[];
-    __shared__ int rowI[kGatherRowsMax * 16];
-    __shared__ float rowG[kGatherRowsMax * 16];
-    __shared__ unsigned rowMask[kGatherRowsMax];
-    __shared__ int s_lo[HOUGH_MAX_LAYERS], s_len[HOUGH_MAX_LAYERS], s_a[HOUGH_MAX_LAYERS];
-    __shared__ int s_total[HOUGH_MAX_LAYERS], s_first[HOUGH_MAX_LAYERS], s_fbase[HOUGH_MAX_LAYERS];
-    __shared__ unsigned s_staged;
-    const Axes &ax = p.ax;
-    const Workspace &w = p.w;
-    const int e = blockIdx.x / p.tiles_per_event;
-    const int t = blockIdx.x - e * p.tiles_per_event;
-    const int rt = t / p.col_tiles, ct = t - rt * p.col_tiles;
-    const int i0 = rt * p.rows, c0 = ct * p.cols;
-    const int nrows = min(p.rows, ax.n_qpt - i0);
-    const int C = p.cols, L = ax.n_layers, nphi = ax.n_phi;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int wcap = count_win_cap(C);
-    int *bpre = reinterpret_cast<int *>(count_smem);          // L slots of wcap + 1 bucket offsets
-    float *fs = reinterpret_cast<float *>(bpre + L * (wcap + 1));   // fcap f values, layer after layer
-    const int64_t hstart = w.hit_start[e];
-    const float *fsort = w.fsort + hstart;
-    const int32_t *offs = w.offs + (int64_t)e * (n_keys(ax) + 1);
-
-    for (int q = threadIdx.x; q < ((p.rows * 16 + 31) & ~31); q += TPB) {
-        const int rr = q >> 4, l = q & 15, i = i0 + rr;
-        int I = 0;
-        float g = 0.f;
-        unsigned valid = 0u;
-        if (l < L && rr < nrows) {
-            const LayerInfo li = w.info[l];
-            const TabEntry te = w.tab[l * ax.n_qpt + i];   // requested with the layer record: one round trip
-            if (li.present && li.uniform && i >= li.lo && i <= li.hi) {
-                if (te.I != kNoVote) {
-                    I = te.I;
-                    g = te.g;
-                    valid = 1u;
-                }
-            }
-        }
-        const unsigned m = __ballot_sync(0xFFFFFFFFu, valid) >> (threadIdx.x & 16);
-        rowI[q] = I;
-        rowG[q] = g;
-        if ((threadIdx.x & 15) == 0) rowMask[rr] = m & 0xFFFFu;
-    }
-    __syncthreads();
-    // each layer's window: buckets [c0 + min I, c0 + C + max I] over the rows it votes on
-    if (threadIdx.x < HOUGH_MAX_LAYERS) {
-        const int l = threadIdx.x;
-        int lo = INT_MAX, hi = INT_MIN, len = 0, a = 0, total = 0, first = 0;
-        if (l < L) {
-            for (int rr = 0; rr < nrows; ++rr)
-                if ((rowMask[rr] >> l) & 1u) {
-                    lo = min(lo, rowI[rr * 16 + l]);
-                    hi = max(hi, rowI[rr * 16 + l]);
-                }
-            if (lo <= hi) {
-                len = C + 2 + (hi - lo);   // buckets J' and J' + 1 of every cell
-                a = wrap_col(c0 + lo, nphi);
-                if (len <= wcap && len <= nphi) {   // one pass over the ring at most
-                    const int32_t *lofs = offs + l * nphi;
-                    const int end = a + len;          // unwrapped end bucket
-                    first = end <= nphi ? lofs[end] - lofs[a] : lofs[nphi] - lofs[a];
-                    total = first + (end <= nphi ? 0 : lofs[end - nphi] - lofs[0]);
-                } else {
-                    len = -len;   // not staged
-                }
-            }
-        }
-        s_lo[l] = lo;
-        s_len[l] = len;
-        s_a[l] = a;
-        s_total[l] = total;
-        s_first[l] = first;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned staged = 0u;
-        int fbase = 0;
-        for (int l = 0; l < L; ++l) {
-            s_fbase[l] = fbase;
-            if (s_len[l] > 0 && fbase + s_total[l] <= fcap) {
-                staged |= 1u << l;
-                fbase += s_total[l];
-            }
-        }
-        s_staged = staged;
-    }
-    __syncthreads();
-    const unsigned staged = s_staged;
-    // staging: every staged layer's bucket offsets (relative to its f values) and f values
-    for (int l = 0; l < L; ++l) {
-        if (!((staged >> l) & 1u)) continue;
-        const int32_t *lofs = offs + l * nphi;
-        const int a = s_a[l], len = s_len[l], first = s_first[l], total = s_total[l], fb = s_fbase[l];
-        int *bp = bpre + l * (wcap + 1);
-        for (int q = threadIdx.x; q <= len; q += TPB) {
-            const int J = a + q;   // unwrapped
-            bp[q] = fb + (J <= nphi ? lofs[J] - lofs[a] : first + lofs[J - nphi] - lofs[0]);
-        }
-        for (int q = threadIdx.x; q < total; q += TPB)
-            fs[fb + q] = q < first ? fsort[lofs[a] + q] : fsort[lofs[0] + (q - first)];
-    }
-    __syncthreads();
-    // a lane per cell, 32 cells of one row per warp pass, every layer summed in a register
-    uint16_t *M = w.M + (int64_t)e * ax.n_qpt * nphi;
-    const int per_row = C >> 5;
-    for (int task = warp; task < nrows * per_row; task += TPB / 32) {
-        const int rr = task / per_row;
-        const int c = (task - rr * per_row) * 32 + lane;
-        const unsigned vm = rowMask[rr];
-        uint32_t count = 0;
-        for (int l = 0; l < L; ++l) {
-            if (!((vm >> l) & 1u)) continue;   // the same for the whole warp: the row's layers
-            const int I = rowI[rr * 16 + l];
-            const float g = rowG[rr * 16 + l];
-            if ((staged >> l) & 1u) {
-                const int *bp = bpre + l * (wcap + 1) + (c + I - s_lo[l]);   // bucket J' of the window
-                const int s0 = bp[0], s1 = bp[1], s2 = bp[2];
-                for (int q = s0; q < s1; ++q) count += fs[q] < g ? 0u : 1u;
-                for (int q = s1; q < s2; ++q) count += fs[q] < g ? 1u : 0u;
-            } else {
-                const int32_t *lofs = offs + l * nphi;
-                const int J0 = wrap_col(c0 + c + I, nphi), J1 = wrap_col(c0 + c + I + 1, nphi);
-                for (int q = lofs[J0]; q < lofs[J0 + 1]; ++q) count += fsort[q] < g ? 0u : 1u;
-                for (int q = lofs[J1]; q < lofs[J1 + 1]; ++q) count += fsort[q] < g ? 1u : 0u;
-            }
-        }
-        // saturated to 16 bits; even lanes store their cell and the next one as one word
-        const uint32_t v = min(count, 65535u);
-        const uint32_t next = __shfl_down_sync(0xFFFFFFFFu, v, 1);
-        if (!(lane & 1))
-            *reinterpret_cast<uint32_t *>(M + (int64_t)(i0 + rr) * nphi + c0 + c) = v | (next << 16);
-    }
-}
-
 // A context's bucket profile is read for the last time by the vote, which the peak search follows:
 // zero it here for the next event (Workspace::recycle).
 __device__ __forceinline__ void recycle_profile(const Axes &ax, const Workspace &w)
@@ -1884,19 +1713,6 @@ cudaError_t launch_scatter_tpb(const VoteParams &p, int threads, size_t smem, in
 
 }  // namespace
 
-// Bucket-offset slots of every layer, then the f values (at least 16 KB, the rest of the budget).
-static size_t gather_count_base_bytes(const Axes &ax, const Tiling &t)
-{
-    return (size_t)ax.n_layers * (count_win_cap(t.gather_cols) + 1) * 4;
-}
-
-size_t gather_count_smem_bytes(const Axes &ax, const Tiling &t)
-{
-    const size_t base = gather_count_base_bytes(ax, t);
-    const size_t fbytes = base + 16384 > (size_t)kCountSmemBudget ? 16384 : (size_t)kCountSmemBudget - base;
-    return base + fbytes;
-}
-
 // Shared memory of the scatter kernel: the column-major tile, the slab's table rows and q/pT centres,
 // then a 32-hit buffer and a queue of FP64 votes per warp.  wide: a 32-bit word a cell.
 static size_t scatter_smem_bytes(const Axes &ax, const Tiling &t, bool wide)
@@ -2044,36 +1860,29 @@ static cudaError_t launch_fused(const Axes &ax, const Workspace &w, const Tiling
     return launch_fused_nl<16>(p, t.gather_threads, smem, blocks, stream);
 }
 
-template <int TPB>
-cudaError_t launch_gather_count_tpb(const GatherParams &p, size_t smem, int fcap, int blocks, cudaStream_t stream)
+// The tile of the shared-atomic vote where the caller's tiling does not choose it (counts in gather mode,
+// the allocation-free vote): 32 rows, a lane each, and as many warps as make the chip busy -- 32 when the
+// tiles do not outnumber the SMs (one 100k-hit event, 128 tiles: 37 us against 45 and 65 us with 16 and 8
+// warps), 8 when there are many, mostly empty ones (16 x 256 x 2048 cells, 1,024 tiles: 33 us against 53
+// us with 32 warps).
+Tiling scatter_tiling(const Axes &ax, int n_events, Tiling t)
 {
-    cudaError_t err = cudaFuncSetAttribute(gather_count_kernel<TPB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)smem);
-    if (err) return err;
-    return launch_chained(gather_count_kernel<TPB>, dim3(blocks), dim3(TPB), smem, stream, p, fcap);
+    t.tile_phi = std::min(ax.n_phi, 256);
+    while (ax.n_phi % t.tile_phi) t.tile_phi -= 64;
+    t.tile_qpt = std::min(ax.n_qpt, 32);
+    const int64_t tiles = (int64_t)n_events * ((ax.n_qpt + t.tile_qpt - 1) / t.tile_qpt) * (ax.n_phi / t.tile_phi);
+    t.threads = tiles <= 152 ? 1024 : tiles <= 608 ? 512 : 256;
+    return t;
 }
 
 cudaError_t launch_gather(const Axes &ax, const Workspace &w, const Tiling &t, cudaStream_t stream)
 {
     if (t.vote_mode == HOUGH_VOTE_FUSED) return launch_fused(ax, w, t, stream);
     if (!ax.counts) return launch_gather_tiled(ax, w, t, stream);
-    if (!w.fsort) return cudaErrorInvalidValue;   // the count gather reads the sorted f values
-    GatherParams p;
-    p.ax = ax;
-    p.w = w;
-    p.rows = t.gather_rows;
-    p.cols = t.gather_cols;
-    p.cap = 0;
-    p.col_tiles = ax.n_phi / p.cols;
-    p.tiles_per_event = ((ax.n_qpt + p.rows - 1) / p.rows) * p.col_tiles;
-    const int blocks = w.n_events * p.tiles_per_event;
-    const size_t smem = gather_count_smem_bytes(ax, t);
-    const int fcap = (int)((smem - gather_count_base_bytes(ax, t)) / 4);
-    switch (t.gather_threads) {
-    case 256: return launch_gather_count_tpb<256>(p, smem, fcap, blocks, stream);
-    case 1024: return launch_gather_count_tpb<1024>(p, smem, fcap, blocks, stream);
-    default: return launch_gather_count_tpb<512>(p, smem, fcap, blocks, stream);
-    }
+    // Counts are scattered in either mode: a cell's count depends on every hit of its buckets, not on two
+    // extrema, and listing them cell by cell took three to fifteen times the scatter's time (100k-hit event
+    // 186 us against 37, 16 x 256 x 2048 cells 628 against 33, 2048 x 2048 with 5,000 hits 342 against 26).
+    return launch_scatter(ax, w, scatter_tiling(ax, w.n_events, t), refine_eps_for(ax), false, stream);
 }
 
 static cudaError_t launch_general(const Axes &ax, const Workspace &w, float refine_eps, cudaStream_t stream)
@@ -2085,17 +1894,16 @@ static cudaError_t launch_general(const Axes &ax, const Workspace &w, float refi
     p.tiles_per_event = ((ax.n_qpt + kGenRows - 1) / kGenRows) * p.n_spans;
     p.s32 = (float)(ax.n_phi * kInvTwoPi);
     p.refine_eps = refine_eps;
-    auto kernel = ax.counts ? general_kernel<true> : general_kernel<false>;
-    cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GeneralSmem));
+    cudaError_t err = cudaFuncSetAttribute(general_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GeneralSmem));
     if (err) return err;
     const int grid = (int)std::min<int64_t>((int64_t)w.n_events * p.tiles_per_event, 152);
-    return launch_chained(kernel, dim3(grid), dim3(kGenThreads), sizeof(GeneralSmem), stream, p);
+    return launch_chained(general_kernel, dim3(grid), dim3(kGenThreads), sizeof(GeneralSmem), stream, p);
 }
 
 cudaError_t launch_scatter(const Axes &ax, const Workspace &w, const Tiling &t, float refine_eps, bool general_only,
                            cudaStream_t stream)
 {
-    if (general_only) return launch_general(ax, w, refine_eps, stream);
+    if (general_only) return ax.counts ? cudaSuccess : launch_general(ax, w, refine_eps, stream);   // (counts: every layer is voted)
     const VoteParams p = vote_params(ax, w, t, refine_eps);
     const int grid = w.n_events * p.tiles_per_event;
     if (ax.counts) {
@@ -2121,7 +1929,7 @@ cudaError_t launch_scatter(const Axes &ax, const Workspace &w, const Tiling &t, 
 cudaError_t launch_vote(const Axes &ax, const Workspace &w, const Tiling &t, float refine_eps,
                         cudaStream_t stream)
 {
-    if (t.vote_mode == HOUGH_VOTE_SCATTER || (ax.counts && !w.fsort)) return launch_scatter(ax, w, t, refine_eps, false, stream);
+    if (t.vote_mode == HOUGH_VOTE_SCATTER) return launch_scatter(ax, w, t, refine_eps, false, stream);
     // gather every table layer (fused with the peak search under HOUGH_VOTE_FUSED), then let the
     // scatter kernel add the layers whose radii differ
     cudaError_t err = launch_gather(ax, w, t, stream);
