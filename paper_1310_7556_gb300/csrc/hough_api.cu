@@ -66,10 +66,9 @@ struct hough_ctx {
     uint8_t *in_layer = nullptr;
     int32_t *mem_idx = nullptr;
     DevStats *stats_host = nullptr;      // pinned
+    DevStats *stats_host_dev = nullptr;  // its device address
     hough_candidate *cands_mapped = nullptr;       // pinned, mapped: hough_process's result staging
     hough_candidate *cands_mapped_dev = nullptr;   // its device address
-    DevStats *stats_mapped = nullptr;              // pinned, mapped: hough_process's counters
-    DevStats *stats_mapped_dev = nullptr;
     int64_t n_hits = 0;
     int stage = 0;                       // 0 nothing, 1 voted, 2 peaks, 3 stage 2
     // counters and radius ranges alternate between two buffers (Workspace::recycle); `clean`: the
@@ -96,7 +95,6 @@ struct hough_ctx {
         for (void *p : allocations) cudaFree(p);
         if (stats_host) cudaFreeHost(stats_host);
         if (cands_mapped) cudaFreeHost(cands_mapped);
-        if (stats_mapped) cudaFreeHost(stats_mapped);
         for (cudaEvent_t e : ev)
             if (e) cudaEventDestroy(e);
     }
@@ -526,7 +524,8 @@ int hough_create(const hough_geometry *geometry, const hough_binning *binning, c
     A(c->alloc(&w.cand_base, 2)); A(c->alloc(&w.counters, 1));
     A(c->alloc(&w.mem_pool, w.max_members)); A(c->alloc(&c->mem_idx, w.max_members));
     A(c->alloc(&c->stats_buf[0], 1)); A(c->alloc(&c->stats_buf[1], 1));
-    A(cudaMallocHost(&c->stats_host, sizeof(DevStats)));
+    A(cudaHostAlloc(reinterpret_cast<void **>(&c->stats_host), sizeof(DevStats), cudaHostAllocMapped));
+    if (e == cudaSuccess) A(cudaHostGetDevicePointer(reinterpret_cast<void **>(&c->stats_host_dev), c->stats_host, 0));
     if (e != cudaSuccess) {
         delete c;
         return cuda_fail(e, "hough_create allocation");
@@ -706,14 +705,19 @@ int hough_get_stats(hough_ctx *c, hough_stats *out, void *stream)
     return HOUGH_OK;
 }
 
-// With host memory the path has one round trip: the hits' per-hit checks run in the staging kernel
-// (the predicates of the host check; a rejected hit makes the call fail with HOUGH_EINVAL once it
-// has synchronised), and the candidates are packed into mapped pinned memory beside the counters'
-// copy, so one synchronisation delivers both.
+// The path has one round trip: one kernel writes the candidates -- into mapped pinned memory, or the
+// caller's device buffer -- and the event's counters into mapped pinned memory, and one synchronisation
+// delivers both (a copy of the counters, a synchronisation, a copy of the candidates they announce and
+// another synchronisation took 10 us more of a 70 us call).  With host memory the hits' per-hit checks
+// run in the staging kernel (the predicates of the host check; a rejected hit makes the call fail with
+// HOUGH_EINVAL once it has synchronised).
 int hough_process(hough_ctx *c, const float *r, const float *phi, const float *z, const uint8_t *layer,
                   int64_t n_hits, hough_candidate *out, int32_t cap, int32_t *n_out, int where, void *stream)
 {
-    if (where != HOUGH_HOST) {
+    const bool host = where == HOUGH_HOST;
+    // (the kernel writes 16-byte vectors)
+    if (!host && (where != HOUGH_DEVICE || !c || !n_out || cap < 0 || (cap > 0 && !out) ||
+                  (reinterpret_cast<uintptr_t>(out) & 15u))) {
         int rc = hough_vote(c, r, phi, z, layer, n_hits, where, stream);
         if (rc) return rc;
         if ((rc = hough_peaks(c, stream))) return rc;
@@ -723,38 +727,32 @@ int hough_process(hough_ctx *c, const float *r, const float *phi, const float *z
     if (!c || !n_out || cap < 0 || (cap > 0 && !out)) return fail(HOUGH_EINVAL, "bad arguments");
     CU(cudaSetDevice(c->device), "cudaSetDevice");
     cudaStream_t s = (cudaStream_t)stream;
-    if (!c->cands_mapped) {   // the first call allocates the staging, once
+    if (host && !c->cands_mapped) {   // the first call allocates the staging, once
         void *h = nullptr, *d = nullptr;
         CU(cudaHostAlloc(&h, sizeof(hough_candidate) * std::max(c->w.max_cand, 1), cudaHostAllocMapped),
            "cudaHostAlloc of the result staging");
         c->cands_mapped = static_cast<hough_candidate *>(h);
         CU(cudaHostGetDevicePointer(&d, h, 0), "cudaHostGetDevicePointer");
         c->cands_mapped_dev = static_cast<hough_candidate *>(d);
-        CU(cudaHostAlloc(&h, sizeof(DevStats), cudaHostAllocMapped), "cudaHostAlloc of the counters");
-        c->stats_mapped = static_cast<DevStats *>(h);
-        CU(cudaHostGetDevicePointer(&d, h, 0), "cudaHostGetDevicePointer");
-        c->stats_mapped_dev = static_cast<DevStats *>(d);
     }
-    int rc = enqueue_vote(c, r, phi, z, layer, n_hits, HOUGH_HOST, s, false);
+    int rc = enqueue_vote(c, r, phi, z, layer, n_hits, where, s, false);
     if (rc) return rc;
     if ((rc = hough_peaks(c, stream))) return rc;
     if ((rc = hough_stage2(c, stream))) return rc;
-    // one kernel writes both the candidates and the counters into mapped memory
-    CU(launch_copy_candidates(c->w, c->cands_mapped_dev, s, std::min<long long>(cap, c->w.max_cand), c->stats_mapped_dev,
-                              152),
+    CU(launch_copy_candidates(c->w, host ? c->cands_mapped_dev : out, s, std::min<long long>(cap, c->w.max_cand),
+                              c->stats_host_dev, 152),
        "copy kernel");
     g_launches += 1;
     CU(cudaStreamSynchronize(s), "synchronise");
-    *c->stats_host = *c->stats_mapped;   // hough_get_stats and friends read the last event's copy
     note_member_cut(c);
     const DevStats &d = *c->stats_host;
-    if (d.device_error & (HOUGH_DEVERR_LAYER | HOUGH_DEVERR_RADIUS))
+    if (host && (d.device_error & (HOUGH_DEVERR_LAYER | HOUGH_DEVERR_RADIUS)))
         return fail(HOUGH_EINVAL, "a hit had layer >= n_layers, r <= 0, |phi| > 1000 or a non-finite coordinate");
     const int64_t found = d.n_candidates;
     const int64_t kept = std::min<int64_t>(found, c->w.max_cand);
     const int64_t ncopy = std::min<int64_t>(kept, cap);
     *n_out = (int32_t)std::min<int64_t>(found, INT32_MAX);
-    if (ncopy > 0) std::memcpy(out, c->cands_mapped, sizeof(hough_candidate) * ncopy);
+    if (host && ncopy > 0) std::memcpy(out, c->cands_mapped, sizeof(hough_candidate) * ncopy);
     if (found > cap) return fail(HOUGH_ETRUNC, "%lld candidates, capacity %d", (long long)found, cap);
     if (found > kept) return fail(HOUGH_ETRUNC, "%lld candidates, max_candidates %d", (long long)found, c->w.max_cand);
     return HOUGH_OK;
