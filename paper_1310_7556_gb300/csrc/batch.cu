@@ -35,6 +35,7 @@ struct hough_batch {
     Axes ax{};
     Tiling tiling{};                     // as a run of n_events uses it: tiling_for
     hough_tiling wanted{};               // as set: a gather tile left open is chosen for each batch size
+    bool by_default = true;              // nothing set: the whole configuration is
     float refine_eps = 0.f;
     hough_batch_limits limits{};
     Workspace w{};
@@ -75,7 +76,14 @@ struct hough_batch {
     }
 
     // The kernel configuration of a run of n events.
-    void tiling_for(int n) { tiling = resolve_tiling(ax, &wanted, n); }
+    void tiling_for(int n)
+    {
+        tiling = by_default ? default_tiling_for(ax, n) : resolve_tiling(ax, &wanted, n);
+        w.band_rows = tiling.band_rows;
+        w.band_cap = band_capacity(ax, tiling.band_rows);
+        w.fused = tiling.vote_mode == HOUGH_VOTE_FUSED;
+        w.use_ranks = w.prank && tiling.vote_mode == HOUGH_VOTE_GATHER;
+    }
 
     // The whole path on the current batch, enqueued on `s` (also the body of the captured graph).
     cudaError_t enqueue(cudaStream_t s)
@@ -111,9 +119,6 @@ int hough_batch_create(const hough_geometry *geometry, const hough_binning *binn
     b->device = device;
     cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, device);
     b->ax = make_axes(geometry, binning);
-    b->tiling = default_tiling_for(b->ax, 1);
-    public_tiling(b->tiling, &b->wanted);
-    b->wanted.gather_rows = b->wanted.gather_cols = b->wanted.gather_threads = 0;
     b->refine_eps = refine_eps_for(b->ax);
     b->limits = *limits;
     const Axes &ax = b->ax;
@@ -154,10 +159,7 @@ int hough_batch_create(const hough_geometry *geometry, const hough_binning *binn
     }
     w.hit_start = b->hit_start;
     w.inputs = b->inputs_dev;
-    w.band_rows = b->tiling.band_rows;
-    w.band_cap = band_capacity(ax, b->tiling.band_rows);
-    w.fused = b->tiling.vote_mode == HOUGH_VOTE_FUSED;
-    w.use_ranks = w.prank && b->tiling.vote_mode == HOUGH_VOTE_GATHER;
+    b->tiling_for(1);
     std::vector<float> kq(ax.n_qpt);
     for (int i = 0; i < ax.n_qpt; ++i) kq[i] = (float)(ax.qpt_min + (i % ax.q_rows + 0.5) * ax.dk);
     A(cudaMemcpy(w.kq32, kq.data(), sizeof(float) * ax.n_qpt, cudaMemcpyHostToDevice));
@@ -184,11 +186,8 @@ int hough_batch_set_tiling(hough_batch *b, const hough_tiling *t)
     int rc = check_tiling_for(b->ax, b->device, t);
     if (rc) return rc;
     b->wanted = *t;
+    b->by_default = false;
     b->tiling_for(1);
-    b->w.band_rows = t->band_rows;
-    b->w.band_cap = band_capacity(b->ax, t->band_rows);
-    b->w.fused = b->tiling.vote_mode == HOUGH_VOTE_FUSED;
-    b->w.use_ranks = b->w.prank && b->tiling.vote_mode == HOUGH_VOTE_GATHER;
     // captured graphs hold the old configuration
     cudaSetDevice(b->device);
     cudaDeviceSynchronize();

@@ -558,9 +558,8 @@ __device__ __forceinline__ int wrap_col(int j, int n)
 // nine neighbours of slice m - 1 precede a cell in raster order (strictly lower), the nine of
 // slice m + 1 follow it (not higher).
 // MASKS: the staged values are the cells' layer masks themselves (compared by their layer counts,
-// and written out from shared memory, M unused).  SMASK: M points to the band's own rows' masks in
-// shared memory (nrows rows of Nphi), not to the accumulator.
-template <int TPB, typename V, bool D3 = false, bool MASKS = false, bool SMASK = false>
+// and written out from shared memory, M unused).
+template <int TPB, typename V, bool D3 = false, bool MASKS = false>
 __device__ __forceinline__ int band_peak_search(const V *pc, int nrows, int i0, int nphi, int threshold,
                                                 const uint16_t *M, uint2 *out, int cap)
 {
@@ -630,9 +629,8 @@ __device__ __forceinline__ int band_peak_search(const V *pc, int nrows, int i0, 
             pk &= pk - 1u;
             if (idx < cap)
                 out[idx] = make_uint2((unsigned)(i0 + rr) << 16 | (unsigned)(j0 + c),
-                                      MASKS   ? (unsigned)pc[(rr + 1) * nphi + j0 + c]
-                                      : SMASK ? (unsigned)M[rr * nphi + j0 + c]
-                                              : (unsigned)M[(int64_t)(i0 + rr) * nphi + j0 + c]);
+                                      MASKS ? (unsigned)pc[(rr + 1) * nphi + j0 + c]
+                                            : (unsigned)M[(int64_t)(i0 + rr) * nphi + j0 + c]);
             ++idx;
         }
         running += s_total;
