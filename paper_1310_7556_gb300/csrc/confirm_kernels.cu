@@ -720,6 +720,7 @@ __device__ __forceinline__ void confirm_groups(const Axes &ax, const Workspace &
             out.mask2 = r_mask2;
             out.flags = ((int)(r_best >> 16) >= min(ax.threshold, ax.n_layers) ? 1u : 0u) | (written < r_members ? 2u : 0u);
             store_candidate(w.cands + f0 + kc, out);
+            if (KEEP && f0 + kc < w.out_limit) store_candidate(w.out_cands + f0 + kc, out);
         }
     }
     flush(0);
@@ -762,40 +763,63 @@ __global__ void __launch_bounds__(32 * kWarps, P10 && !EVENT ? 7 : 5)
         total = (int)w.counters->total_cands;
     }
     const size_t scratch = sizeof(Scratch) + (size_t)start_words * 4;
+    int workers = 1;   // CTAs with candidates
     if (EVENT && total <= kTeamRounds * (int)gridDim.x) {
-        if ((int)blockIdx.x >= total) return;
-        Scratch &S = *reinterpret_cast<Scratch *>(smem_c + warp * scratch);
-        unsigned *starts = reinterpret_cast<unsigned *>(&S + 1);
-        uint32_t *grid = reinterpret_cast<uint32_t *>(smem_c + kWarps * scratch);
-        for (int q = threadIdx.x; q < grid_words >> 2; q += 32 * kWarps)
-            reinterpret_cast<uint4 *>(grid)[q] = make_uint4(0u, 0u, 0u, 0u);
-        __syncthreads();
-        if (general)
-            confirm_groups<NL, P10, G64, true, true, true>(ax, w, s32, refine_eps, S, &s_team, starts, grid, grid_words >> 2, present,
-                                                     general, 1, blockIdx.x, gridDim.x, total, coarse, chunk);
-        else
-            confirm_groups<NL, P10, G64, false, true, true>(ax, w, s32, refine_eps, S, &s_team, starts, grid, grid_words >> 2, present,
-                                                      0u, 1, blockIdx.x, gridDim.x, total, coarse, chunk);
-        return;
+        workers = max(1, min((int)gridDim.x, total));
+        if ((int)blockIdx.x < total) {
+            Scratch &S = *reinterpret_cast<Scratch *>(smem_c + warp * scratch);
+            unsigned *starts = reinterpret_cast<unsigned *>(&S + 1);
+            uint32_t *grid = reinterpret_cast<uint32_t *>(smem_c + kWarps * scratch);
+            for (int q = threadIdx.x; q < grid_words >> 2; q += 32 * kWarps)
+                reinterpret_cast<uint4 *>(grid)[q] = make_uint4(0u, 0u, 0u, 0u);
+            __syncthreads();
+            if (general)
+                confirm_groups<NL, P10, G64, true, true, true>(ax, w, s32, refine_eps, S, &s_team, starts, grid, grid_words >> 2,
+                                                               present, general, 1, blockIdx.x, gridDim.x, total, coarse, chunk);
+            else
+                confirm_groups<NL, P10, G64, false, true, true>(ax, w, s32, refine_eps, S, &s_team, starts, grid,
+                                                                grid_words >> 2, present, 0u, 1, blockIdx.x, gridDim.x, total,
+                                                                coarse, chunk);
+        }
+    } else {
+        // candidates per warp: as many as its lanes hold, fewer when that would leave warps without any;
+        // group q goes to CTA q mod gridDim, so that a few candidates spread over all SMs
+        const int nwarps = group_warps * gridDim.x;
+        const int C = max(1, min(32 / NL, total / nwarps));
+        const int first = warp * gridDim.x + blockIdx.x;
+        workers = max(1, min((int)gridDim.x, (total + C - 1) / C));
+        if (warp < group_warps && (int64_t)first * C < total) {
+            Scratch &S = *reinterpret_cast<Scratch *>(smem_c + warp * (scratch + (size_t)grid_words * 4));
+            unsigned *starts = reinterpret_cast<unsigned *>(&S + 1);
+            uint32_t *grid = starts + start_words;
+            for (int q = lane; q < grid_words >> 2; q += 32) reinterpret_cast<uint4 *>(grid)[q] = make_uint4(0u, 0u, 0u, 0u);
+            __syncwarp();
+            if (general)
+                confirm_groups<NL, P10, G64, true, EVENT, false>(ax, w, s32, refine_eps, S, nullptr, starts, grid,
+                                                                 grid_words >> 2, present, general, C, first, nwarps, total,
+                                                                 coarse, chunk);
+            else
+                confirm_groups<NL, P10, G64, false, EVENT, false>(ax, w, s32, refine_eps, S, nullptr, starts, grid,
+                                                                  grid_words >> 2, present, 0u, C, first, nwarps, total, coarse,
+                                                                  chunk);
+        }
     }
-    // candidates per warp: as many as its lanes hold, fewer when that would leave warps without any;
-    // group q goes to CTA q mod gridDim, so that a few candidates spread over all SMs
-    if (warp >= group_warps) return;
-    const int nwarps = group_warps * gridDim.x;
-    const int C = max(1, min(32 / NL, total / nwarps));
-    const int first = warp * gridDim.x + blockIdx.x;
-    if ((int64_t)first * C >= total) return;
-    Scratch &S = *reinterpret_cast<Scratch *>(smem_c + warp * (scratch + (size_t)grid_words * 4));
-    unsigned *starts = reinterpret_cast<unsigned *>(&S + 1);
-    uint32_t *grid = starts + start_words;
-    for (int q = lane; q < grid_words >> 2; q += 32) reinterpret_cast<uint4 *>(grid)[q] = make_uint4(0u, 0u, 0u, 0u);
-    __syncwarp();
-    if (general)
-        confirm_groups<NL, P10, G64, true, EVENT, false>(ax, w, s32, refine_eps, S, nullptr, starts, grid, grid_words >> 2, present,
-                                                  general, C, first, nwarps, total, coarse, chunk);
-    else
-        confirm_groups<NL, P10, G64, false, EVENT, false>(ax, w, s32, refine_eps, S, nullptr, starts, grid, grid_words >> 2, present,
-                                                   0u, C, first, nwarps, total, coarse, chunk);
+    if (!EVENT || !w.out_stats || (int)blockIdx.x >= workers) return;
+    // the CTA that finishes last of those with candidates (the first, if there are none) reports the
+    // event's counters, complete by then
+    __shared__ int s_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(&w.counters->confirms_done, 1u) == (unsigned)workers - 1u;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    static_assert(sizeof(DevStats) % 4 == 0, "the counters are copied as 32-bit words");
+    for (int q = threadIdx.x; q < (int)(sizeof(DevStats) / 4); q += blockDim.x)
+        reinterpret_cast<uint32_t *>(w.out_stats)[q] = __ldcg(reinterpret_cast<const uint32_t *>(w.stats) + q);
+    if (threadIdx.x == 0) w.counters->confirms_done = 0u;   // ready for the next event
 }
 
 __global__ void member_index_kernel(Workspace w, int32_t *idx_out, int64_t total)

@@ -274,13 +274,12 @@ Tiling default_tiling_impl(const Axes &ax, int n_events)
     if (!ax.counts && !ax.n_d0)
         for (int r : {8, 4, 2})
             if (t.band_rows == 1 && (int64_t)n_events * n_bands(ax, r) >= 512) t.band_rows = r;
-    // with a d0 axis a band stages its rows in three slices: taller bands stage each row fewer times
+    // with a d0 axis a band reads its rows in three slices: taller bands read each row fewer times
     if (ax.n_d0)
-        for (int r : {4, 2})
-            if (band_smem_bytes(ax, r) + 1024 <= 232448) {
+        for (int r : {8, 4, 2})
+            if (t.band_rows == 1 && band_smem_bytes(ax, r) + 1024 <= 232448 &&
+                (r == 2 || (int64_t)n_events * n_bands(ax, r) >= 512 || (ax.counts && r == 4)) && !(ax.counts && r == 8))
                 t.band_rows = r;
-                break;
-            }
     return resolve_tiling_impl(ax, &t, n_events);
 }
 
@@ -711,9 +710,9 @@ int hough_get_stats(hough_ctx *c, hough_stats *out, void *stream)
     return HOUGH_OK;
 }
 
-// The path has one round trip: one kernel writes the candidates -- into mapped pinned memory, or the
-// caller's device buffer -- and the event's counters into mapped pinned memory, and one synchronisation
-// delivers both (a copy of the counters, a synchronisation, a copy of the candidates they announce and
+// The path has one round trip: the confirmation itself writes the candidates also into mapped pinned
+// memory, or the caller's device buffer, and its last CTA the event's counters into mapped pinned memory,
+// and one synchronisation delivers both (a copy of the counters, a synchronisation, a copy of the candidates they announce and
 // another synchronisation took 10 us more of a 70 us call).  With host memory the hits' per-hit checks
 // run in the staging kernel (the predicates of the host check; a rejected hit makes the call fail with
 // HOUGH_EINVAL once it has synchronised).
@@ -744,11 +743,14 @@ int hough_process(hough_ctx *c, const float *r, const float *phi, const float *z
     int rc = enqueue_vote(c, r, phi, z, layer, n_hits, where, s, false);
     if (rc) return rc;
     if ((rc = hough_peaks(c, stream))) return rc;
-    if ((rc = hough_stage2(c, stream))) return rc;
-    CU(launch_copy_candidates(c->w, host ? c->cands_mapped_dev : out, s, std::min<long long>(cap, c->w.max_cand),
-                              c->stats_host_dev, 152),
-       "copy kernel");
-    g_launches += 1;
+    c->w.out_cands = host ? c->cands_mapped_dev : out;
+    c->w.out_limit = std::min<long long>(cap, c->w.max_cand);
+    c->w.out_stats = c->stats_host_dev;
+    rc = hough_stage2(c, stream);
+    c->w.out_cands = nullptr;
+    c->w.out_limit = 0;
+    c->w.out_stats = nullptr;
+    if (rc) return rc;
     CU(cudaStreamSynchronize(s), "synchronise");
     note_member_cut(c);
     const DevStats &d = *c->stats_host;

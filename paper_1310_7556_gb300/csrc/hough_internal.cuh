@@ -135,7 +135,8 @@ struct HitInputs {
 struct BatchCounters {
     unsigned int total_cands;      // candidates kept over all events
     unsigned int scans_done;       // events whose band counts are scanned (the last one's CTA adds up the totals)
-    unsigned int pad[2];
+    unsigned int confirms_done;    // CTAs of the confirmation that have finished (the last one reports the counters)
+    unsigned int pad;
 };
 
 // Device buffers of a batch of events that share one set of axes.
@@ -186,6 +187,11 @@ struct Workspace {
     int copy_wait;                // < 0: the first bound on a bulk-copy wait expires at once (a test of the error path)
     int cands_from_bands;         // one event: the confirmation reads its candidates from the band lists
     int n_band_lists;             // their number (set with it)
+    // one event of a context: the confirmation also writes the first out_limit records to out_cands and,
+    // once every CTA is done, the event's counters to out_stats (device-accessible; null: it does not)
+    hough_candidate *out_cands;
+    long long out_limit;
+    DevStats *out_stats;
     // A context's state is left clean for its next event by the kernels that last use it, so that no
     // clearing kernel opens the next event: the hit sort zeroes the bucket counts, the peak search
     // the bucket profile, and the counting kernel the counters and radius ranges of the next event,
@@ -247,10 +253,8 @@ cudaError_t launch_band_peaks(const Axes &ax, const Workspace &w, const Tiling &
 // The band lists into cand_list, the candidate counts and cand_base.  records: also write the
 // candidates' records with the stage-2 fields empty (a caller reads them before stage 2).
 cudaError_t launch_compact(const Axes &ax, const Workspace &w, cudaStream_t stream, bool records = false);
-// The first `limit` candidate records into `out` (device-accessible); the first event's counters to
-// `stats_out` (device-accessible) when it is given.
-cudaError_t launch_copy_candidates(const Workspace &w, hough_candidate *out, cudaStream_t stream, long long limit,
-                                   DevStats *stats_out = nullptr, int blocks = 1216);
+// The first `limit` candidate records into `out` (device-accessible).
+cudaError_t launch_copy_candidates(const Workspace &w, hough_candidate *out, cudaStream_t stream, long long limit);
 cudaError_t launch_stage2(const Axes &ax, const Workspace &w, int sms, float refine_eps, cudaStream_t stream,
                           cudaEvent_t between = nullptr);
 cudaError_t launch_member_index(const Workspace &w, int32_t *idx_out, int64_t total, cudaStream_t stream);

@@ -29,7 +29,7 @@
 // Peaks: candidates of each band of band_rows rows (one row by default) go to a band list in
 // raster order; a scan of the band counts and a copy then concatenate the band lists of all events
 // into one list.
-// With a d0 axis a band lies in one slice and its cells take the 3 x 3 x 3 rule (peaks3_kernel).
+// With a d0 axis a band lies in one slice and its cells take the 3 x 3 x 3 rule (peaks_mask_kernel<true>, peaks3_count_kernel).
 #include <algorithm>
 #include <atomic>
 #include <climits>
@@ -1511,20 +1511,26 @@ __host__ __device__ inline size_t peak_smem_bytes(int band_rows, int nphi)
     return (size_t)band_rows * peak_segments(nphi) * (32 + sizeof(int));
 }
 
+// D3: a grid with a d0 axis.  A band is band_rows q/pT rows of one slice m, and a cell's 3 x 3 x 3 block adds
+// the maxima of its nine neighbours in slice m - 1, which precede it in raster order (strictly lower), and in
+// slice m + 1 (not higher); rows outside the slice and slices outside the grid are empty.
+template <bool D3>
 __global__ void __launch_bounds__(kPeakThreads) peaks_mask_kernel(Axes ax, Workspace w)
 {
     pdl_enter();
     recycle_profile(ax, w);
-    if (w.fused && all_layers_uniform(ax, w)) return;   // the fused vote searched the bands
+    if (!D3 && w.fused && all_layers_uniform(ax, w)) return;   // the fused vote searched the bands
     extern __shared__ __align__(16) unsigned char pc[];
     __shared__ int s_warp[kPeakThreads / 32];
     const int R = w.band_rows, nphi = ax.n_phi;
     const int nb = n_bands(ax, R), nseg = peak_segments(nphi);
     const int e = blockIdx.x / nb, band = blockIdx.x - e * nb;
-    const int i0 = band * R, nrows = min(R, ax.n_qpt - i0);
+    const int Q = ax.q_rows;                                     // rows of a slice
+    const int bps = (Q + R - 1) / R, m = D3 ? band / bps : 0;    // bands of a slice, the band's slice
+    const int i0 = (band - m * bps) * R, nrows = min(R, Q - i0);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int NW = kPeakThreads / 32;
-    const uint16_t *M = w.M + (int64_t)e * ax.n_qpt * nphi;
+    const uint16_t *M = w.M + ((int64_t)e * ax.n_qpt + (int64_t)m * Q) * nphi;   // the band's slice
     unsigned char *flags = pc;                                   // [row][segment][lane]
     int *seg_n = reinterpret_cast<int *>(pc + (size_t)R * nseg * 32);   // [row][segment]
     const unsigned thr = (unsigned)ax.threshold | (unsigned)ax.threshold << 16;
@@ -1535,11 +1541,11 @@ __global__ void __launch_bounds__(kPeakThreads) peaks_mask_kernel(Axes ax, Works
         // the column before the first lane's, or after the last lane's (phi wraps)
         const int jh = lane == 0 ? (j0 ? j0 - 1 : nphi - 1) : (j0 + 8 < nphi ? j0 + 8 : 0);
         const bool halo_lane = lane == 0 || lane == last;
-        auto load = [&](int i, uint4 &v, unsigned &halo) {
+        auto load = [&](int i, uint4 &v, unsigned &halo, int slice = 0) {   // slice: -1, 0, 1 of the band's
             v = make_uint4(0u, 0u, 0u, 0u);
             halo = 0u;
-            if (i >= 0 && i < ax.n_qpt) {
-                const uint16_t *row = M + (int64_t)i * nphi;
+            if (i >= 0 && i < Q && (!D3 || (m + slice >= 0 && m + slice < ax.n_d0))) {
+                const uint16_t *row = M + (int64_t)(i + slice * Q) * nphi;
                 if (on) v = *reinterpret_cast<const uint4 *>(row + j0);
                 if (halo_lane) halo = row[jh];
             }
@@ -1557,15 +1563,51 @@ __global__ void __launch_bounds__(kPeakThreads) peaks_mask_kernel(Axes ax, Works
         PeakRow cur = peak_row(v[1], halo[1], lane, last);
         uint4 vn = v[2];
         unsigned hn = halo[2];
+        // the slices before and after: their rows' maxima of three columns, the last two rows
+        unsigned before[2][4], after[2][4];
+        uint4 vb, va;
+        unsigned hb, ha;
+        if (D3) {
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                load(i0 - 1 + q, vb, hb, -1);
+                load(i0 - 1 + q, va, ha, 1);
+                const PeakRow rb = peak_row(vb, hb, lane, last), ra = peak_row(va, ha, lane, last);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    before[q][k] = rb.h[k];
+                    after[q][k] = ra.h[k];
+                }
+            }
+            load(i0 + 1, vb, hb, -1);
+            load(i0 + 1, va, ha, 1);
+        }
         for (int r = 0; r < nrows; ++r) {
             const PeakRow dn = peak_row(vn, hn, lane, last);
             if (r + 1 < nrows) load(i0 + r + 2, vn, hn);
+            PeakRow rb, ra;
+            if (D3) {
+                rb = peak_row(vb, hb, lane, last);
+                ra = peak_row(va, ha, lane, last);
+                if (r + 1 < nrows) {
+                    load(i0 + r + 2, vb, hb, -1);
+                    load(i0 + r + 2, va, ha, 1);
+                }
+            }
             unsigned f = 0u;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 // counts are at most 16: no carry between the halves
-                const unsigned need = __vmaxu2(__vmaxu2(__vmaxu2(up[k], cur.left[k]) + 0x00010001u, thr),
-                                               __vmaxu2(dn.h[k], cur.right[k]));
+                unsigned lower = __vmaxu2(up[k], cur.left[k]), upper = __vmaxu2(dn.h[k], cur.right[k]);
+                if (D3) {
+                    lower = __vmaxu2(lower, __vmaxu2(__vmaxu2(before[0][k], before[1][k]), rb.h[k]));
+                    upper = __vmaxu2(upper, __vmaxu2(__vmaxu2(after[0][k], after[1][k]), ra.h[k]));
+                    before[0][k] = before[1][k];
+                    before[1][k] = rb.h[k];
+                    after[0][k] = after[1][k];
+                    after[1][k] = ra.h[k];
+                }
+                const unsigned need = __vmaxu2(__vmaxu2(lower + 0x00010001u, thr), upper);
                 const unsigned ge = ((cur.p[k] | 0x80008000u) - need) & 0x80008000u;   // p >= need, by halves
                 f |= (ge >> 15 & 1u) << (2 * k) | (ge >> 31) << (2 * k + 1);
             }
@@ -1624,7 +1666,8 @@ __global__ void __launch_bounds__(kPeakThreads) peaks_mask_kernel(Axes ax, Works
         while (f) {
             const int c = __ffs(f) - 1;
             f &= f - 1u;
-            if (at < w.band_cap) out[at] = make_uint2((unsigned)i << 16 | (unsigned)(j0 + c), M[(int64_t)i * nphi + j0 + c]);
+            if (at < w.band_cap)
+                out[at] = make_uint2((unsigned)(m * Q + i) << 16 | (unsigned)(j0 + c), M[(int64_t)i * nphi + j0 + c]);
             ++at;
         }
     }
@@ -1659,17 +1702,16 @@ __global__ void __launch_bounds__(kPeakThreads) peaks_count_kernel(Axes ax, Work
     if (threadIdx.x == 0) w.band_counts[(int64_t)e * nb + band] = cnt;
 }
 
-// Peak search of one band of band_rows q/pT rows of one d0 slice m of a grid with a d0 axis: the
-// rows of its cells' 3 x 3 x 3 blocks -- rows i0 - 1 .. i0 + nrows of slices m - 1, m, m + 1 --
-// are staged as cell values (layer counts as bytes, or 16-bit counts), rows outside the slice and
-// slices outside the grid as empty.  Bands never cross a slice, so the band lists concatenate in
-// raster order.
-template <bool COUNTS>
-__global__ void __launch_bounds__(kPeakThreads) peaks3_kernel(Axes ax, Workspace w)
+// Peak search of one band of band_rows q/pT rows of one d0 slice m of a grid of vote counts with a d0 axis:
+// the rows of its cells' 3 x 3 x 3 blocks -- rows i0 - 1 .. i0 + nrows of slices m - 1, m, m + 1 -- are staged
+// as they are, rows outside the slice and slices outside the grid as empty.  Bands never cross a slice, so
+// the band lists concatenate in raster order.
+__global__ void __launch_bounds__(kPeakThreads) peaks3_count_kernel(Axes ax, Workspace w)
 {
     pdl_enter();
     recycle_profile(ax, w);
     extern __shared__ __align__(16) unsigned char pc[];
+    uint16_t *pv = reinterpret_cast<uint16_t *>(pc);
     const int R = w.band_rows, Q = ax.q_rows;
     const int bps = (Q + R - 1) / R;   // bands per slice
     const int nb = n_bands(ax, R);
@@ -1687,29 +1729,11 @@ __global__ void __launch_bounds__(kPeakThreads) peaks3_kernel(Axes ax, Workspace
         uint4 v = make_uint4(0u, 0u, 0u, 0u);
         if (mm >= 0 && mm < ax.n_d0 && ii >= 0 && ii < Q)
             v = *reinterpret_cast<const uint4 *>(M + (int64_t)(mm * Q + ii) * nphi + c8 * 8);
-        if (COUNTS) {
-            *reinterpret_cast<uint4 *>(reinterpret_cast<uint16_t *>(pc) + sidx * nphi + c8 * 8) = v;
-        } else {
-            const uint32_t words[4] = {v.x, v.y, v.z, v.w};
-            uint32_t packed[2] = {0u, 0u};
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint32_t lo = (uint32_t)__popc(words[u] & 0xFFFFu), hi = (uint32_t)__popc(words[u] >> 16);
-                packed[u >> 1] |= (lo | (hi << 8)) << ((u & 1) * 16);
-            }
-            *reinterpret_cast<uint2 *>(pc + sidx * nphi + c8 * 8) = make_uint2(packed[0], packed[1]);
-        }
+        *reinterpret_cast<uint4 *>(pv + sidx * nphi + c8 * 8) = v;
     }
     __syncthreads();
     uint2 *out = w.band_cands + ((int64_t)e * nb + band) * w.band_cap;
-    const int row0 = m * Q + i0;   // stacked row of the band's first row
-    int cnt;
-    if (COUNTS)
-        cnt = band_peak_search<kPeakThreads, uint16_t, true>(reinterpret_cast<const uint16_t *>(pc), nrows, row0, nphi,
-                                                             ax.threshold, M, out, w.band_cap);
-    else
-        cnt = band_peak_search<kPeakThreads, unsigned char, true>(pc, nrows, row0, nphi, ax.threshold, M, out,
-                                                                  w.band_cap);
+    const int cnt = band_peak_search<kPeakThreads, uint16_t, true>(pv, nrows, m * Q + i0, nphi, ax.threshold, M, out, w.band_cap);
     if (threadIdx.x == 0) w.band_counts[(int64_t)e * nb + band] = cnt;
 }
 
@@ -1809,18 +1833,11 @@ __global__ void __launch_bounds__(256) band_copy_kernel(Axes ax, Workspace w, in
     }
 }
 
-// The first `limit` candidate records of all events to `out`, 16 bytes a thread.  When `stats_out` is
-// given, block 0 also copies the first event's counters there.
-__global__ void copy_candidates_kernel(Workspace w, hough_candidate *out, long long limit, DevStats *stats_out)
+// The first `limit` candidate records of all events to `out`, 16 bytes a thread.
+__global__ void copy_candidates_kernel(Workspace w, hough_candidate *out, long long limit)
 {
     pdl_enter();
-    static_assert(sizeof(DevStats) % 4 == 0, "the counters are copied as 32-bit words");
     static_assert(sizeof(hough_candidate) == 32, "a record is two 16-byte vectors");
-    if (stats_out && blockIdx.x == 0) {
-        const uint32_t *src = reinterpret_cast<const uint32_t *>(w.stats);
-        uint32_t *dst = reinterpret_cast<uint32_t *>(stats_out);
-        for (int q = threadIdx.x; q < (int)(sizeof(DevStats) / 4); q += blockDim.x) dst[q] = src[q];
-    }
     const long long n = 2 * min((long long)w.cand_base[w.n_events], limit);
     const uint4 *src = reinterpret_cast<const uint4 *>(w.cands);
     uint4 *dst = reinterpret_cast<uint4 *>(out);
@@ -2079,10 +2096,9 @@ cudaError_t launch_vote(const Axes &ax, const Workspace &w, const Tiling &t, flo
 cudaError_t launch_band_peaks(const Axes &ax, const Workspace &w, const Tiling &t, cudaStream_t stream)
 {
     const int nb = n_bands(ax, w.band_rows);
-    const bool masks = !ax.counts && !ax.n_d0;
-    const size_t smem = masks ? peak_smem_bytes(w.band_rows, ax.n_phi) : band_smem_bytes(ax, w.band_rows);
-    auto kernel = ax.n_d0 ? (ax.counts ? peaks3_kernel<true> : peaks3_kernel<false>)
-                          : (ax.counts ? peaks_count_kernel : peaks_mask_kernel);
+    const size_t smem = ax.counts ? band_smem_bytes(ax, w.band_rows) : peak_smem_bytes(w.band_rows, ax.n_phi);
+    auto kernel = ax.n_d0 ? (ax.counts ? peaks3_count_kernel : peaks_mask_kernel<true>)
+                          : (ax.counts ? peaks_count_kernel : peaks_mask_kernel<false>);
     cudaError_t err;
     if ((err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return err;
     if ((err = launch_chained(kernel, dim3(w.n_events * nb), dim3(kPeakThreads), smem, stream, ax, w))) return err;
@@ -2098,10 +2114,9 @@ cudaError_t launch_compact(const Axes &ax, const Workspace &w, cudaStream_t stre
     return launch_chained(band_copy_kernel, dim3(blocks), dim3(256), 0, stream, ax, w, records ? 1 : 0);
 }
 
-cudaError_t launch_copy_candidates(const Workspace &w, hough_candidate *out, cudaStream_t stream, long long limit,
-                                   DevStats *stats_out, int blocks)
+cudaError_t launch_copy_candidates(const Workspace &w, hough_candidate *out, cudaStream_t stream, long long limit)
 {
-    return launch_chained(copy_candidates_kernel, dim3(blocks), dim3(256), 0, stream, w, out, limit, stats_out);
+    return launch_chained(copy_candidates_kernel, dim3(1216), dim3(256), 0, stream, w, out, limit);
 }
 
 }  // namespace hough

@@ -39,3 +39,13 @@ def test_saturated_grid(binding, n_layers):
         bn = eg.Binning(n_qpt=24, qpt_min=-1.0, qpt_max=1.0, n_phi=512, threshold=1)
     ev = eg.simulate_event(geo, 0, (1.0, 50.0), 1500 * n_layers, seed=5)
     check_event(binding, geo, bn, ev)
+
+
+@pytest.mark.parametrize("band_rows", [1, 2, 5, 16])
+@pytest.mark.parametrize("n_qpt, n_phi, n_d0, threshold", [(1, 64, 1, 2), (7, 128, 3, 4), (18, 704, 2, 5), (5, 512, 9, 3)])
+def test_bands_of_a_d0_grid(binding, band_rows, n_qpt, n_phi, n_d0, threshold):
+    geo = eg.Geometry()
+    bn = eg.Binning(n_qpt=n_qpt, qpt_min=-0.8, qpt_max=0.8, n_phi=n_phi, threshold=threshold, n_d0=n_d0, d0_min=-1.5,
+                    d0_max=1.5)
+    ev = eg.simulate_event(geo, 40, (1.5, 50.0), 300, seed=n_qpt + n_phi, d0_range=(-1.5, 1.5))
+    check_event(binding, geo, bn, ev, tiling=dict(band_rows=band_rows))
