@@ -83,6 +83,7 @@ struct hough_batch {
         w.band_cap = band_capacity(ax, tiling.band_rows);
         w.fused = tiling.vote_mode == HOUGH_VOTE_FUSED;
         w.use_ranks = w.prank && tiling.vote_mode == HOUGH_VOTE_GATHER;
+        w.slim = !ax.counts && tiling.vote_mode != HOUGH_VOTE_SCATTER;
     }
 
     // The whole path on the current batch, enqueued on `s` (also the body of the captured graph).

@@ -825,9 +825,9 @@ __global__ void __launch_bounds__(32 * kWarps, P10 && !EVENT ? 7 : 5)
 __global__ void member_index_kernel(Workspace w, int32_t *idx_out, int64_t total)
 {
     pdl_enter();
-    const ColdHit *cold = w.cold + w.hit_start[0];
+    const int32_t *isort = w.isort + w.hit_start[0];
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x)
-        idx_out[q] = cold[w.mem_pool[q]].idx;
+        idx_out[q] = isort[w.mem_pool[q]];
 }
 
 // Words of a grid of 16-bit masks, two to a word, or of 10-bit masks, three to a word, rounded up

@@ -380,6 +380,7 @@ int enqueue_vote(hough_ctx *c, const float *r, const float *phi, const float *z,
     c->w.band_cap = band_capacity(c->ax, c->tiling.band_rows);
     c->w.fused = c->tiling.vote_mode == HOUGH_VOTE_FUSED;
     c->w.use_ranks = c->w.prank && c->tiling.vote_mode == HOUGH_VOTE_GATHER;
+    c->w.slim = !c->ax.counts && c->tiling.vote_mode != HOUGH_VOTE_SCATTER;
     if (c->timing) { CU(cudaEventRecord(c->ev[0], s), "event"); c->timed |= 1 | (0xF << 8); }
     // this event's counters and radius ranges; the other buffer of each is zeroed for the next one
     c->w.stats = c->stats_buf[c->parity];
@@ -515,7 +516,7 @@ int hough_create(const hough_geometry *geometry, const hough_binning *binning, c
         A(c->alloc(&w.prank, (size_t)prof_event_entries(ax)));
         A(c->alloc(&w.gsort, (size_t)ax.n_layers * ax.n_qpt)); A(c->alloc(&w.rankt, (size_t)ax.n_layers * ax.n_qpt));
     }
-    A(c->alloc(&w.hot, n)); A(c->alloc(&w.cold, n)); A(c->alloc(&w.fsort, n)); A(c->alloc(&w.zsort, n));
+    A(c->alloc(&w.hot, n)); A(c->alloc(&w.cold, n)); A(c->alloc(&w.fsort, n)); A(c->alloc(&w.zsort, n)); A(c->alloc(&w.isort, n));
     A(c->alloc(&c->radii_buf[0], 1)); A(c->alloc(&c->radii_buf[1], 1));
     A(c->alloc(&w.info, HOUGH_MAX_LAYERS)); A(c->alloc(&w.memo, 1));
     A(c->alloc(&w.tab, (size_t)ax.n_layers * ax.n_qpt));

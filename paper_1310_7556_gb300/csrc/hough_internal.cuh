@@ -159,7 +159,10 @@ struct Workspace {
     HotHit *hot;                  // per hit, sorted within each event's range
     float *fsort;                 // per hit, sorted: the hot record's f alone (count gather, membership)
     float *zsort;                 // per hit, sorted: z alone (membership; may be null when no stage 2 runs)
+    int32_t *isort;               // per hit, sorted: index in the caller's arrays (contexts: member lists; may be null)
     ColdHit *cold;
+    int slim;                     // 1: no kernel reads the hot and cold records of a layer of one radius (the gather
+                                  // reads bucket profiles, the confirmation f and z): the sort leaves them out
     LayerRadii *radii;            // batch-wide
     LayerInfo *info;              // HOUGH_MAX_LAYERS
     TableMemo *memo;              // (null: the table is computed for every event, by table_chunks CTAs a layer)

@@ -488,15 +488,24 @@ __device__ __forceinline__ void recycle_counts(const Axes &ax, const Workspace &
     for (int64_t q = n / 4 * 4 + t0; q < n; q += nthreads) w.counts[q] = 0;
 }
 
-// Valid hit h (input index; event start `start`) to its sorted position pos: its f, hot record hh
-// completed with its voting rows, cold record (r, phi, z) and z.
-__device__ __forceinline__ void sort_hit(const Axes &ax, const Workspace &w, int64_t h, int e, int64_t start,
-                                         int64_t pos, HotHit hh, float rr, float ph, float zz, int e0,
+// Valid hit h (input index; event start `start`) to its sorted position pos: its f, z and index, and --
+// unless its layer has one radius and nothing reads them (Workspace::slim) -- its hot record hh completed
+// with its voting rows and its cold record (r, phi, z).  Leaving the two 16-byte records out saves two of
+// the three or four memory sectors a hit's scattered stores touch.
+__device__ __forceinline__ void sort_hit(const Axes &ax, const Workspace &w, const HitInputs &in, int64_t h, int e,
+                                         int64_t start, int64_t pos, HotHit hh, float rr, float ph, float zz, int e0,
                                          unsigned *s_votes)
 {
     if (w.fsort) w.fsort[pos] = hh.f;
+    if (w.zsort) w.zsort[pos] = zz;
+    if (w.isort) w.isort[pos] = (int32_t)(h - start);
     const int l = (hh.jl >> 16) & 0xF;
     const LayerInfo li = w.info[l];
+    if (w.slim) {
+        if (li.uniform) return;
+        rr = in.r[h];
+        ph = in.phi[h];
+    }
     int lo = li.lo, hi = li.hi;
     if (!li.uniform && ax.n_d0) {
         // every row may hold a vote; the vote kernels decide each in FP64
@@ -526,7 +535,6 @@ __device__ __forceinline__ void sort_hit(const Axes &ax, const Workspace &w, int
     ch.z = zz;
     ch.idx = (int32_t)(h - start);
     w.cold[pos] = ch;
-    if (w.zsort) w.zsort[pos] = ch.z;
 }
 
 // The rank form of a bucket profile entry (see kRankRows), by thread t0 of nthreads: a layer of one
@@ -584,9 +592,11 @@ __global__ void __launch_bounds__(kStageThreads) hit_sort_kernel(Axes ax, Worksp
         k = w.key[t0];
         rank = w.rank[t0];
         hh = w.hot_tmp[t0];
-        rr = in.r[t0];
-        ph = in.phi[t0];
         zz = in.z[t0];
+        if (!w.slim) {
+            rr = in.r[t0];
+            ph = in.phi[t0];
+        }
     }
     __shared__ unsigned s_votes[HOUGH_MAX_LAYERS];
     if (threadIdx.x < HOUGH_MAX_LAYERS) s_votes[threadIdx.x] = 0u;
@@ -613,13 +623,15 @@ __global__ void __launch_bounds__(kStageThreads) hit_sort_kernel(Axes ax, Worksp
             k = w.key[h];
             rank = w.rank[h];
             hh = w.hot_tmp[h];
-            rr = in.r[h];
-            ph = in.phi[h];
             zz = in.z[h];
+            if (!w.slim) {
+                rr = in.r[h];
+                ph = in.phi[h];
+            }
         }
         const int e = event_of(w.hit_start, w.n_events, h);
         const int64_t start = w.hit_start[e];
-        if (k >= 0) sort_hit(ax, w, h, e, start, start + w.offs[(int64_t)e * (nkeys + 1) + k] + rank, hh, rr, ph, zz, e0, s_votes);
+        if (k >= 0) sort_hit(ax, w, in, h, e, start, start + w.offs[(int64_t)e * (nkeys + 1) + k] + rank, hh, rr, ph, zz, e0, s_votes);
     }
     if (t0 < npairs && tli.present && tli.uniform && tli.nvote > 0 && tn)
         atomicAdd(&w.stats[te].votes_by_layer[tl], (unsigned long long)tn * (unsigned long long)tli.nvote);
