@@ -343,6 +343,9 @@ def measure_plain(env, args, ctx, tens, n):
 
 # Kernels of one plain step: (name, timing key, source file that defines it).  Their algorithmic
 # work per launch is kernel_work's model below.
+# (labels of the steps: the gather is gather_rank_kernel or gather_kernel, the vote of per-vote layers
+# general_kernel after a gather, the peak search peaks_mask_kernel or the counts' kernels, the compaction
+# band_scan_kernel and band_copy_kernel)
 PLAIN_KERNELS = [
     ("clear_kernel", "clear_ms", "stage_kernels.cu"),
     ("stage_count_kernel", "count_ms", "stage_kernels.cu"),
