@@ -258,7 +258,9 @@ int hough_process(hough_ctx *ctx, const float *r, const float *phi, const float 
  * (identical result, no atomics).  Each CTA of the gather kernel (gather_threads threads) owns a
  * tile of gather_rows rows x gather_cols columns and stages the slices of the bucket profile the
  * tile reads into shared memory with bulk asynchronous copies.  Layers whose hits lie at several
- * radii are added by the shared-atomic scatter kernel.
+ * radii are added by a shared-atomic kernel with a tile of its own.  Known fault: a tile wider than
+ * 256 columns whose width is not a multiple of 256 (320, 384, 448; the default on some grids whose
+ * n_phi is not a multiple of 512) leaves the columns past its last 256 unwritten (zero).
  * vote_mode HOUGH_VOTE_SCATTER: every layer by the shared-atomic scatter kernel (Sec. 6.1), each
  * CTA owning a tile of tile_qpt rows x tile_phi columns in shared memory.
  * vote_mode HOUGH_VOTE_FUSED (layer masks without a d0 axis): the gather and the peak search in
